@@ -940,6 +940,10 @@ dc_status dc_render_viewport(dc_ctx *ctx, int n_vp, const dc_viewport *vps, void
         d.width = vp.width;
         d.height = vp.height;
         d.offset = off;
+        d.dxh = (float)d.dx;
+        d.dxl = (float)(d.dx - (double)d.dxh);
+        d.dyh = (float)d.dy;
+        d.dyl = (float)(d.dy - (double)d.dyh);
         vl.push_back(d);
         off += np;
     }

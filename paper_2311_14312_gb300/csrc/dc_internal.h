@@ -172,6 +172,7 @@ struct VpDev {
     double x0, y0, dx, dy;
     int width, height;
     long long offset;         // first output pixel of this viewport
+    float dxh, dxl, dyh, dyl; // dx, dy as FP32 (hi, lo) pairs
 };
 
 // Exclusive scan of int counts on the device (aa.cu): out[i] = sum of

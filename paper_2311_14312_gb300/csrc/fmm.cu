@@ -180,11 +180,11 @@ __device__ __forceinline__ unsigned char q8(double v) {
     return (unsigned char)floor(255.0 * v + 0.5);
 }
 
-__global__ void eval_tiles_kernel(DevTree t, const Tile *__restrict__ tiles, const VpDev *__restrict__ vps, int P1,
+__global__ void eval_tiles_kernel(DevTree t, const RTile *__restrict__ tiles, const VpDev *__restrict__ vps, int P1,
                                   const double2 *__restrict__ M, const double2 *__restrict__ L,
                                   const double *__restrict__ sbar, const double *__restrict__ mbar,
                                   void *rgb, int rgb_dtype, unsigned char *rgb8) {
-    Tile tl = tiles[blockIdx.x];
+    const RTile tl = tiles[blockIdx.x];
     const VpDev vp = vps[tl.vp];
     int npx = tl.nr * tl.nc;
     for (int j = threadIdx.x; j < npx; j += blockDim.x) {
@@ -1758,16 +1758,17 @@ dc_status Fmm::render_viewports(const VpDev *vpl, int n_vp, const double *sbar, 
     // the plan is built here while the stream runs the passes before the
     // render; its upload is ordered after them on the stream
     I.plan_valid = false;
-    std::vector<Tile> tiles;
+    std::vector<RTile> tiles;
     std::vector<double> cost;   // estimated flops per tile
-    int TW = kEvalTile, TH = kEvalTile;
-    if (I.fp32) tile_shape(I.opt.eval_tile, TW, TH);
     long long pairs = 0;
     const long long m2p0 = I.render_m2p;
     const double flops0 = I.render_flops;
     for (int v = 0; v < n_vp; ++v) {
         const VpDev &vp = vpl[v];
         if (vp.width == 0 || vp.height == 0) continue;
+        const long long vpx = (long long)vp.width * vp.height;
+        int cap_w = kEvalTile, cap_h = kEvalTile;
+        if (I.fp32) tile_cap(I.opt.eval_tile, vpx, cap_w, cap_h);
         for (int c = 0; c < T.n_cells(); ++c) {
             if (!T.is_leaf(c)) continue;
             double w = T.width(c);
@@ -1783,11 +1784,23 @@ dc_status Fmm::render_viewports(const VpDev *vpl, int n_vp, const double *sbar, 
             long long wn = T.w_ptr[c + 1] - T.w_ptr[c];
             I.render_m2p += wn * npx;
             I.render_flops += 45.0 * double(up * npx) + 24.0 * I.P1 * double((1 + wn) * npx);
+            const int TW = tile_side(w / vp.dx, cap_w), TH = tile_side(w / vp.dy, cap_h);
             for (int r = r0; r < r1; r += TH)
                 for (int cc = c0; cc < c1; cc += TW) {
-                    tiles.push_back({c, r, cc, std::min(TH, r1 - r), std::min(TW, c1 - cc), v});
+                    RTile q{c, r, cc, std::min(TH, r1 - r), std::min(TW, c1 - cc), v, 0, 0, 0, 0, 0, 0};
+                    const double x = vp.x0 + (q.c0 + 0.5 * q.nc) * vp.dx, y = vp.y0 + (q.r0 + 0.5 * q.nr) * vp.dy;
+                    q.cxh = (float)x;
+                    q.cxl = (float)(x - (double)q.cxh);
+                    q.cyh = (float)y;
+                    q.cyl = (float)(y - (double)q.cyh);
+                    q.tx = (float)(x - T.cx(c));
+                    q.ty = (float)(y - T.cy(c));
+                    tiles.push_back(q);
                     const double tp = double(std::min(TH, r1 - r)) * std::min(TW, c1 - cc);
-                    cost.push_back(tp * (45.0 * double(up) + 24.0 * I.P1 * double(1 + wn)));
+                    // sampled rectangles: the samples, a share of the pieces and the polynomial
+                    const double direct = 45.0 * double(up) + 24.0 * I.P1 * double(1 + wn);
+                    const bool sampled = I.fp32 && tp > 48.0 && w >= 15.0 * std::max(vp.dx, vp.dy);
+                    cost.push_back(sampled ? 32.0 * direct + tp * (100.0 + 8.0 * double(up)) : tp * direct);
                 }
         }
     }
@@ -1804,7 +1817,7 @@ dc_status Fmm::render_viewports(const VpDev *vpl, int n_vp, const double *sbar, 
             cnt[bin[i] + 1]++;
         }
         for (int b = 0; b < kBins; ++b) cnt[b + 1] += cnt[b];
-        std::vector<Tile> sorted(tiles.size());
+        std::vector<RTile> sorted(tiles.size());
         for (size_t i = 0; i < tiles.size(); ++i) sorted[cnt[bin[i]]++] = tiles[i];
         tiles.swap(sorted);
     }

@@ -34,7 +34,6 @@ __device__ __forceinline__ float2 fmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 __device__ __forceinline__ float2 fadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 fscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 __device__ __forceinline__ float2 finv(float2 a) {
     float d = 1.0f / (a.x * a.x + a.y * a.y);
     return make_float2(a.x * d, -a.y * d);
@@ -166,13 +165,17 @@ __global__ void near_centre_kernel(const int *__restrict__ uf_ptr, const int *__
     }
 }
 
-template <typename From, typename To>
-__global__ void narrow_kernel(const From *__restrict__ a, To *__restrict__ b, size_t n) {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        b[i].x = (float)a[i].x;
-        b[i].y = (float)a[i].y;
-    }
+// FP32 copies of the expansions for the evaluation: M with M_k / k in the
+// place of M_k (k >= 1), the factor of Eq. 61, and L.
+__global__ void narrow_kernel(const double2 *__restrict__ M, const double2 *__restrict__ L, float2 *__restrict__ M32,
+                              float2 *__restrict__ L32, int P1, size_t n) {
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int k = (int)(i % P1);
+    const float ik = k > 0 ? 1.f / k : 1.f;
+    const double2 m = M[i], l = L[i];
+    M32[i] = make_float2((float)m.x * ik, (float)m.y * ik);
+    L32[i] = make_float2((float)l.x, (float)l.y);
 }
 
 // heavy[i] = 1 when max_c |sigma_bar| w len or |mu_bar| w len of piece i
@@ -193,26 +196,17 @@ __global__ void heavy_kernel(const double *__restrict__ sb, const double *__rest
 }
 
 // -------------------------------------------------------------- eval --
-// The pixel tile of one block is TW x TH pixels (options.eval_tile picks
-// the shape); every shape is compiled for the same resident threads per SM
-// (kEvThreadsPerSM), so the register budget does not depend on the shape.
-// resident blocks per SM of 64-thread tiles the register budget is set for,
-// and pieces staged in shared memory per round
-#ifndef DC_EVAL_MINBLOCKS
-#define DC_EVAL_MINBLOCKS 12
-#endif
-#ifndef DC_EVAL_STAGE
-#define DC_EVAL_STAGE 128
-#endif
-constexpr int kEvBlocksPerSM = DC_EVAL_MINBLOCKS;
-constexpr int kEvThreadsPerSM = 64 * kEvBlocksPerSM;
-
-constexpr int kStage = DC_EVAL_STAGE;
+// Arbitrary points (render_viewport's pixels: rendertiles.cuh): one block of
+// 64 threads per item of up to 64 points of one leaf; resident blocks per SM
+// the register budget is set for, and pieces staged in shared memory per round
+constexpr int kEvBlocksPerSM = 12;
+constexpr int kStage = 128;
 
 struct EvalArgs32 {
     DevTree32 t;
     DevTree t64;
-    const Tile *items;
+    const Tile *items;     // list mode
+    const RTile *rects;    // pixel mode
     int P1;
     const float2 *M, *L;
     const float *sb, *mb;
@@ -260,7 +254,6 @@ __device__ __forceinline__ void split2(double v, float &hi, float &lo) {
     lo = (float)(v - (double)hi);
 }
 
-template <int MODE, int TW, int TH>
 __device__ __forceinline__ void eval32_item(const EvalArgs32 &a, int item) {
     // staged pieces of one list-1 leaf, in the target leaf's frame, each
     // coordinate as a (hi, lo) float pair so differences keep full accuracy
@@ -278,27 +271,15 @@ __device__ __forceinline__ void eval32_item(const EvalArgs32 &a, int item) {
     const int j = threadIdx.x;
     bool act;
     double qx64 = 0.0, qy64 = 0.0;
-    int own1 = -1, own2 = -1, r = 0, c = 0, ti = 0;
-    VpDev vp;
-    if (MODE == 0) {
-        vp = a.vps[tl.vp];
-        act = j < tl.nr * tl.nc;
-        if (act) {
-            r = tl.r0 + j / tl.nc;
-            c = tl.c0 + j % tl.nc;
-            qx64 = vp.x0 + (c + 0.5) * vp.dx;
-            qy64 = vp.y0 + (r + 0.5) * vp.dy;
-        }
-    } else {
-        act = j < tl.nr;
-        if (act) {
-            ti = tl.r0 + j;
-            qx64 = a.q64[2 * ti];
-            qy64 = a.q64[2 * ti + 1];
-            if (a.own1) {
-                own1 = a.own1[ti];
-                own2 = a.own2[ti];
-            }
+    int own1 = -1, own2 = -1, ti = 0;
+    act = j < tl.nr;
+    if (act) {
+        ti = tl.r0 + j;
+        qx64 = a.q64[2 * ti];
+        qy64 = a.q64[2 * ti + 1];
+        if (a.own1) {
+            own1 = a.own1[ti];
+            own2 = a.own2[ti];
         }
     }
     float qxh, qxl, qyh, qyl;
@@ -366,13 +347,11 @@ __device__ __forceinline__ void eval32_item(const EvalArgs32 &a, int item) {
             float2 iz = finv(zz);
             float lz = 0.5f * __logf(zz.x * zz.x + zz.y * zz.y) + t.logw[src];
             const float2 *Ms = a.M + (size_t)src * 3 * P1;
-            float2 m0 = fscale(Ms[P1 - 1], 1.f / (P1 - 1)), m1 = fscale(Ms[2 * P1 - 1], 1.f / (P1 - 1)),
-                   m2 = fscale(Ms[3 * P1 - 1], 1.f / (P1 - 1));
+            float2 m0 = Ms[P1 - 1], m1 = Ms[2 * P1 - 1], m2 = Ms[3 * P1 - 1];   // M_k / k
             for (int k = P1 - 2; k >= 1; --k) {
-                float ik = 1.f / k;
-                m0 = fadd(fmul(m0, iz), fscale(Ms[k], ik));
-                m1 = fadd(fmul(m1, iz), fscale(Ms[P1 + k], ik));
-                m2 = fadd(fmul(m2, iz), fscale(Ms[2 * P1 + k], ik));
+                m0 = fadd(fmul(m0, iz), Ms[k]);
+                m1 = fadd(fmul(m1, iz), Ms[P1 + k]);
+                m2 = fadd(fmul(m2, iz), Ms[2 * P1 + k]);
             }
             m0 = fmul(m0, iz);
             m1 = fmul(m1, iz);
@@ -524,43 +503,17 @@ __device__ __forceinline__ void eval32_item(const EvalArgs32 &a, int item) {
         }
     }
     if (!act) return;
-    if (MODE == 0) {
-        size_t o = 3 * ((size_t)vp.offset + (size_t)r * vp.width + c);
-        float u[3] = {(float)(u0 + h0), (float)(u1 + h1), (float)(u2 + h2)};
-        for (int ch = 0; ch < 3; ++ch) {
-            if (a.rgb) {
-                if (a.rgb_dtype == DC_F64) static_cast<double *>(a.rgb)[o + ch] = (double)u[ch];
-                else static_cast<float *>(a.rgb)[o + ch] = u[ch];
-            }
-            if (a.rgb8) a.rgb8[o + ch] = quant8(u[ch]);
-        }
-    } else {
-        int o = a.perm[ti];
-        a.out[3 * (size_t)o + 0] = u0 + h0;
-        a.out[3 * (size_t)o + 1] = u1 + h1;
-        a.out[3 * (size_t)o + 2] = u2 + h2;
-    }
+    const int o = a.perm[ti];
+    a.out[3 * (size_t)o + 0] = u0 + h0;
+    a.out[3 * (size_t)o + 1] = u1 + h1;
+    a.out[3 * (size_t)o + 2] = u2 + h2;
 }
 
-// One item per block, or, with a.queue, a persistent grid whose blocks take
-// items from the counter *a.queue in list order (the render's tiles are
-// listed by decreasing estimated cost, so the longest start first).
-template <int MODE, int TW, int TH>
-__global__ void __launch_bounds__(TW * TH, kEvThreadsPerSM / (TW * TH)) eval32_kernel(EvalArgs32 a) {
-    if (!a.queue) {
-        eval32_item<MODE, TW, TH>(a, blockIdx.x);
-        return;
-    }
-    __shared__ int next;
-    while (true) {
-        __syncthreads();
-        if (threadIdx.x == 0) next = atomicAdd(a.queue, 1);
-        __syncthreads();
-        const int it = next;
-        if (it >= a.n_items) break;
-        eval32_item<MODE, TW, TH>(a, it);
-    }
+__global__ void __launch_bounds__(64, kEvBlocksPerSM) eval32_kernel(EvalArgs32 a) {
+    eval32_item(a, blockIdx.x);
 }
+
+#include "rendertiles.cuh"
 
 // ----------------------------------------------------- host helpers --
 using cd = std::complex<double>;
@@ -885,9 +838,8 @@ cudaError_t Fmm::Impl::prepare_render32(const double *sb, const double *mb, cuda
     big_coef_kernel<<<(unsigned)(((size_t)nC * 32 + th - 1) / th), th, 0, st>>>(L.ptr, M.ptr, nC, P1, heavyL.ptr, heavyM.ptr);
     note_launch();
     const size_t n = (size_t)nC * 3 * P1;
-    narrow_kernel<double2, float2><<<(unsigned)((n + th - 1) / th), th, 0, st>>>(M.ptr, M32.ptr, n);
-    narrow_kernel<double2, float2><<<(unsigned)((n + th - 1) / th), th, 0, st>>>(L.ptr, L32.ptr, n);
-    note_launch(2);
+    narrow_kernel<<<(unsigned)((n + th - 1) / th), th, 0, st>>>(M.ptr, L.ptr, M32.ptr, L32.ptr, P1, n);
+    note_launch();
     return cudaGetLastError();
 }
 
@@ -1101,7 +1053,7 @@ cudaError_t Fmm::Impl::render_tiles32(int n_tiles, void *rgb, int rgb_dtype,
 
     a.t = dt32();
     a.t64 = dt();
-    a.items = tiles.ptr;
+    a.rects = tiles.ptr;
     a.P1 = P1;
     a.M = M32.ptr;
     a.L = L32.ptr;
@@ -1117,23 +1069,14 @@ cudaError_t Fmm::Impl::render_tiles32(int n_tiles, void *rgb, int rgb_dtype,
     a.rgb = rgb;
     a.rgb_dtype = rgb_dtype;
     a.rgb8 = rgb8;
-    // persistent: as many blocks as are resident (the same register budget
-    // for every tile shape), taking tiles from a counter
+    // persistent: as many blocks as are resident, taking rectangles from a counter
     cudaError_t e;
     if ((e = render_queue.ensure(1)) != cudaSuccess ||
         (e = cudaMemsetAsync(render_queue.ptr, 0, sizeof(int), st)) != cudaSuccess)
         return e;
     a.queue = render_queue.ptr;
     a.n_items = n_tiles;
-    int tw = 8, th = 8;
-    tile_shape(opt.eval_tile, tw, th);
-    const int grid = std::max(1, std::min(n_tiles, n_sms * (kEvThreadsPerSM / (tw * th))));
-    switch (opt.eval_tile) {   // tile shapes of tile_shape()
-    case 1: eval32_kernel<0, 16, 8><<<grid, 128, 0, st>>>(a); break;
-    case 2: eval32_kernel<0, 16, 16><<<grid, 256, 0, st>>>(a); break;
-    case 3: eval32_kernel<0, 32, 8><<<grid, 256, 0, st>>>(a); break;
-    default: eval32_kernel<0, 8, 8><<<grid, 64, 0, st>>>(a); break;
-    }
+    rtiles::render32_kernel<<<std::min(n_tiles, n_sms * rtiles::kBlocksPerSM), 32 * rtiles::kWarps, 0, st>>>(a);
     note_launch();
     return cudaGetLastError();
 }
@@ -1169,7 +1112,7 @@ cudaError_t Fmm::Impl::eval_points32_at(const Tile *items, int n_items, const do
     a.q64 = q64;
     a.perm = perm;
     a.out = out;
-    eval32_kernel<1, 8, 8><<<n_items, 64, 0, st>>>(a); note_launch();
+    eval32_kernel<<<n_items, 64, 0, st>>>(a); note_launch();
     return cudaGetLastError();
 }
 

@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -52,18 +53,41 @@ struct Tile {
     int leaf, r0, c0, nr, nc, vp;   // vp: viewport index (pixel tiles)
 };
 
-// Pixel tiles of the render: kEvalTile x kEvalTile pixels of one leaf per
-// block of the evaluation kernel, one thread per pixel.
-#ifndef DC_EVAL_TILE
-#define DC_EVAL_TILE 8
-#endif
-constexpr int kEvalTile = DC_EVAL_TILE;
-// pixel tile width x height of the FP32 evaluation kernel for options.eval_tile
-inline void tile_shape(int eval_tile, int &w, int &h) {
-    static const int W[4] = {8, 16, 16, 32}, H[4] = {8, 8, 16, 8};
-    const int k = (eval_tile >= 0 && eval_tile < 4) ? eval_tile : 0;
-    w = W[k];
-    h = H[k];
+// A rectangle of the render with its centre: in world units as FP32 (hi, lo)
+// pairs, and relative to the leaf's centre (computed with the plan: FP64 work
+// on the device costs 64 times FP32's).
+struct RTile {
+    int leaf, r0, c0, nr, nc, vp;
+    float cxh, cxl, cyh, cyl, tx, ty;
+};
+
+// Pixel rectangles of the FP64 form's render: kEvalTile x kEvalTile pixels
+// of one leaf per block of the evaluation kernel, one thread per pixel.
+constexpr int kEvalTile = 8;
+
+// The FP32 form's render (rendertiles.cuh): the largest rectangle, in pixels
+// a side, in a viewport of px pixels (it has to leave enough rectangles to
+// fill the GPU); options.eval_tile 1..3 caps it at 16 x 8, 16 x 16, 32 x 8.
+// 64 x 64 was slower at every size (24 viewports of 87 Mpixels: 18.9 against
+// 17.6 ms): what it saves on samples its near pieces cost again.
+inline void tile_cap(int eval_tile, long long px, int &w, int &h) {
+    static const int W[4] = {0, 16, 16, 32}, H[4] = {0, 8, 16, 8};
+    w = h = px >= 500000 ? 32 : px >= 250000 ? 16 : 8;
+    if (eval_tile >= 1 && eval_tile <= 3) {
+        w = std::min(w, W[eval_tile]);
+        h = std::min(h, H[eval_tile]);
+    }
+}
+// Side of the rectangles in a leaf of `pixels` pixels a side: a power of two
+// in [8, cap], half the leaf at most (the circle around a rectangle then
+// stays clear of what the leaf's local expansion stands for), and past 16 an
+// eighth: a wider one's near zone, 2.5 times its radius, would hold the pieces
+// of the neighbouring leaves (a quarter: 2.23 against 1.92 ms on a 1021 x 613
+// window).
+inline int tile_side(double pixels, int cap) {
+    int s = 8;
+    while (2 * s <= cap && (s < 16 ? 2.0 : 8.0) * 2 * s <= pixels) s *= 2;
+    return s;
 }
 
 // Cells that need incoming expansions for one set of targets (all cells for
@@ -146,7 +170,7 @@ struct Fmm::Impl {
     // FP64 tables and expansions
     DevBuf<double2> m2m, l2l, m2l, M, L;
     DevBuf<double> sbar, mbar;
-    DevBuf<Tile> tiles;               // the render's tiles, by decreasing estimated cost
+    DevBuf<RTile> tiles;              // the render's tiles, by decreasing estimated cost
     DevBuf<int> render_queue;         // the persistent render's tile counter
     DevBuf<VpDev> vps;
     // FP32 form
