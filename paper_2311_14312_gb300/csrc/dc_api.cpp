@@ -1002,8 +1002,8 @@ dc_status dc_render_viewport(dc_ctx *ctx, int n_vp, const dc_viewport *vps, void
                                                    ctx->aa.n_samples, ctx->aa.u.ptr, s),
                       "anti-aliasing samples");
             } else {
-                dc_status fs = ctx->fmm->eval_points_dev(ctx->aa.sxy.ptr, ctx->aa.n_samples, ctx->sbar.ptr,
-                                                         ctx->mbar.ptr, ctx->aa.u.ptr, s, msg);
+                dc_status fs = ctx->fmm->sort_points(ctx->aa.sxy.ptr, ctx->aa.n_samples, s, msg);
+                if (fs == DC_OK) fs = ctx->fmm->eval_sorted(ctx->sbar.ptr, ctx->mbar.ptr, ctx->aa.u.ptr, s, msg);
                 if (fs != DC_OK) return fail(ctx, fs, msg);
             }
             DC_CK(ctx, ctx->aa.finish(drgb, rgb_dtype, drgb8, s), "anti-aliasing");
@@ -1102,10 +1102,16 @@ dc_status dc_eval_points(dc_ctx *ctx, int n, const void *xy, int xy_where, void 
               "outputs");
     } else {
         std::string msg;
-        DC_CK(ctx, ctx->fmm->prepare_eval(ctx->sbar.ptr, ctx->mbar.ptr, s), "fmm passes");
-        dc_status fs =
-            ctx->fmm->eval_points(dxy, n, ctx->sbar.ptr, ctx->mbar.ptr, dout, out_dtype, s, msg);
+        // the sort first: its wait is then not for the passes, and what
+        // follows is queued without a gap (sorting on the host cost 11.4 ms
+        // for 100,003 points, the kernels take 1.4)
+        dc_status fs = ctx->fmm->sort_points(dxy, n, s, msg);
         if (fs != DC_OK) return fail(ctx, fs, msg);
+        DC_CK(ctx, ctx->u64.ensure(size_t(3) * n), "alloc");
+        DC_CK(ctx, ctx->fmm->prepare_eval(ctx->sbar.ptr, ctx->mbar.ptr, s), "fmm passes");
+        fs = ctx->fmm->eval_sorted(ctx->sbar.ptr, ctx->mbar.ptr, ctx->u64.ptr, s, msg);
+        if (fs != DC_OK) return fail(ctx, fs, msg);
+        DC_CK(ctx, dc::launch_write_outputs(ctx->u64.ptr, n, dout, out_dtype, nullptr, s), "outputs");
     }
     if (out_where == DC_MEM_HOST) {
         DC_CK(ctx, cudaMemcpyAsync(out, dout, size_t(3) * n * esz, cudaMemcpyDeviceToHost, s),

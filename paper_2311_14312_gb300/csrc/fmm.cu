@@ -1843,100 +1843,34 @@ dc_status Fmm::render_viewports(const VpDev *vpl, int n_vp, const double *sbar, 
 }
 
 
-dc_status Fmm::eval_points(const double *xy, int n, const double *sbar, const double *mbar,
-                           void *out, int out_dtype, cudaStream_t st, std::string &err) {
+dc_status Fmm::sort_points(const double *xy, int n, cudaStream_t st, std::string &err) {
     Impl &I = *impl_;
+    I.n_pt_items = 0;
+    if (n <= 0) return DC_OK;
     const Tree &T = I.tree;
-    std::vector<double> h(2 * size_t(n));
-    cudaError_t e = cudaMemcpyAsync(h.data(), xy, h.size() * sizeof(double), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    bool outside = false;
+    const int item = I.fp32 ? 64 : evalnodes::kNodeItem;
+    const cudaError_t e = I.psort.run(xy, n, I.child0.ptr, I.cc.ptr, T.n_cells(), T.x0, T.y0, T.w0, item, I.fp32, st,
+                                      I.n_pt_items, outside);
     if (e != cudaSuccess) {
-        err = cudaGetErrorString(e);
-        return DC_ERR_CUDA;
-    }
-    const int nC = T.n_cells();
-    std::vector<int> leaf_of(n), cnt(nC, 0);
-    for (int i = 0; i < n; ++i) {
-        int lf = T.locate(h[2 * i], h[2 * i + 1]);
-        if (lf < 0) {
-            err = "eval_points: point outside the quadtree root; widen options.domain";
-            return DC_ERR_ARG;
-        }
-        leaf_of[i] = lf;
-        cnt[lf]++;
-    }
-    std::vector<int> start(nC), perm(n), leaves;
-    std::vector<double> sxy(2 * size_t(n));
-    for (int c = 0, acc = 0; c < nC; ++c) {
-        start[c] = acc;
-        acc += cnt[c];
-        if (cnt[c]) leaves.push_back(c);
-    }
-    std::vector<int> fill(start);
-    for (int i = 0; i < n; ++i) {
-        int j = fill[leaf_of[i]]++;
-        perm[j] = i;
-        sxy[2 * j] = h[2 * i];
-        sxy[2 * j + 1] = h[2 * i + 1];
-    }
-    if ((e = upload(I.pt_leaves, leaves, st)) != cudaSuccess || (e = upload(I.pt_start, start, st)) != cudaSuccess ||
-        (e = upload(I.pt_count, cnt, st)) != cudaSuccess || (e = upload(I.pt_perm, perm, st)) != cudaSuccess ||
-        (e = upload(I.pt_xy, sxy, st)) != cudaSuccess || (e = I.pt_out.ensure(3 * size_t(n))) != cudaSuccess) {
         err = cudaGetErrorString(e);
         return e == cudaErrorMemoryAllocation ? DC_ERR_OOM : DC_ERR_CUDA;
     }
-    if (I.fp32) {
-        std::vector<Tile> items;
-        std::vector<float2> q32(n);
-        for (int c : leaves) {
-            double cx = T.cx(c), cy = T.cy(c);
-            for (int j = start[c]; j < start[c] + cnt[c]; ++j)
-                q32[j] = make_float2((float)(sxy[2 * j] - cx), (float)(sxy[2 * j + 1] - cy));
-            for (int j = 0; j < cnt[c]; j += 64) items.push_back({c, start[c] + j, 0, std::min(64, cnt[c] - j), 0, 0});
-        }
-        if ((e = upload(I.pt_items, items, st)) != cudaSuccess || (e = upload(I.pt_q32, q32, st)) != cudaSuccess ||
-            (e = I.eval_points32(int(items.size()), I.pt_out.ptr, sbar, mbar, st)) != cudaSuccess) {
-            err = cudaGetErrorString(e);
-            return DC_ERR_CUDA;
-        }
-    } else {
-        std::vector<int4> items4;
-        for (int c : leaves)
-            for (int j = 0; j < cnt[c]; j += evalnodes::kNodeItem)
-                items4.push_back(make_int4(c, start[c] + j, std::min(evalnodes::kNodeItem, cnt[c] - j), 0));
-        if ((e = upload(I.pt_items4, items4, st)) != cudaSuccess ||
-            (e = I.eval_list64(I.pt_items4.ptr, int(items4.size()), I.pt_xy.ptr, nullptr, nullptr,
-                               I.pt_perm.ptr, sbar, mbar, 1, 1, I.pt_out.ptr, st)) != cudaSuccess) {
-            err = cudaGetErrorString(e);
-            return DC_ERR_CUDA;
-        }
-    }
-    if ((e = launch_write_outputs(I.pt_out.ptr, n, out, out_dtype, nullptr, st)) != cudaSuccess) {
-        err = cudaGetErrorString(e);
-        return DC_ERR_CUDA;
+    if (outside) {
+        err = "eval_points: point outside the quadtree root; widen options.domain";
+        return DC_ERR_ARG;
     }
     return DC_OK;
 }
 
-dc_status Fmm::eval_points_dev(const double *xy, int n, const double *sbar, const double *mbar, double *out,
-                               cudaStream_t st, std::string &err) {
+dc_status Fmm::eval_sorted(const double *sbar, const double *mbar, double *out, cudaStream_t st, std::string &err) {
     Impl &I = *impl_;
-    if (n <= 0) return DC_OK;
-    const Tree &T = I.tree;
-    int n_items = 0;
-    bool outside = false;
-    const int item = I.fp32 ? 64 : evalnodes::kNodeItem;
-    cudaError_t e = I.psort.run(xy, n, I.child0.ptr, I.cc.ptr, T.n_cells(), T.x0, T.y0, T.w0, item, I.fp32, st,
-                                n_items, outside);
-    if (e == cudaSuccess && outside) {
-        err = "eval_points: point outside the quadtree root; widen options.domain";
-        return DC_ERR_ARG;
-    }
-    if (e == cudaSuccess)
-        e = I.fp32 ? I.eval_points32_at(I.psort.items32.ptr, n_items, I.psort.sxy.ptr, I.psort.perm.ptr, out, sbar,
-                                        mbar, st)
-                   : I.eval_list64(I.psort.items64.ptr, n_items, I.psort.sxy.ptr, nullptr, nullptr,
-                                   I.psort.perm.ptr, sbar, mbar, 1, 1, out, st);
+    if (I.n_pt_items == 0) return DC_OK;
+    const cudaError_t e =
+        I.fp32 ? I.eval_points32_at(I.psort.items32.ptr, I.n_pt_items, I.psort.sxy.ptr, I.psort.perm.ptr, out, sbar,
+                                    mbar, st)
+               : I.eval_list64(I.psort.items64.ptr, I.n_pt_items, I.psort.sxy.ptr, nullptr, nullptr, I.psort.perm.ptr,
+                               sbar, mbar, 1, 1, out, st);
     if (e != cudaSuccess) {
         err = cudaGetErrorString(e);
         return e == cudaErrorMemoryAllocation ? DC_ERR_OOM : DC_ERR_CUDA;

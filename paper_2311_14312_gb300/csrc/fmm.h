@@ -55,7 +55,7 @@ public:
                       cudaStream_t st, GmresResult &res, std::string &err, int *n_refine = nullptr,
                       const double *Ax0 = nullptr);
     // Forms the expansions of segment densities sbar and mbar (Alg. 8 up and
-    // down passes); render_grid / eval_points then evaluate them.
+    // down passes); render_viewports / eval_sorted then evaluate them.
     cudaError_t prepare_eval(const double *sbar, const double *mbar, cudaStream_t st);
     // Single + double layer of segment densities at the pixels of n
     // viewports in one launch; rgb / rgb8 are the outputs of the whole call
@@ -63,13 +63,12 @@ public:
     dc_status render_viewports(const VpDev *vps, int n, const double *sbar, const double *mbar,
                                void *rgb, int rgb_dtype, unsigned char *rgb8, cudaStream_t st,
                                std::string &err);
-    dc_status eval_points(const double *xy, int n, const double *sbar, const double *mbar,
-                          void *out, int out_dtype, cudaStream_t st, std::string &err);
-    // The same at device points xy [n][2], FP64 output out [n][3], with the
-    // points located and sorted by leaf on the device (no host round trip);
-    // after prepare_eval.
-    dc_status eval_points_dev(const double *xy, int n, const double *sbar, const double *mbar, double *out,
-                              cudaStream_t st, std::string &err);
+    // Arbitrary device points xy [n][2]: sort_points locates and sorts them by
+    // leaf on the device (one wait, for the number of work items and whether
+    // a point lies outside the root), eval_sorted evaluates them into out
+    // [n][3] (FP64, the caller's order) after prepare_eval.
+    dc_status sort_points(const double *xy, int n, cudaStream_t st, std::string &err);
+    dc_status eval_sorted(const double *sbar, const double *mbar, double *out, cudaStream_t st, std::string &err);
     void fill_sizes(dc_sizes *out) const;
     // wall ms of the build phases: tree and lists, schedules and uploads,
     // preconditioner, stored P2M / P2L rows, near / far coefficients, FP32 form

@@ -1081,11 +1081,6 @@ cudaError_t Fmm::Impl::render_tiles32(int n_tiles, void *rgb, int rgb_dtype,
     return cudaGetLastError();
 }
 
-cudaError_t Fmm::Impl::eval_points32(int n_items, double *out, const double *sb64,
-                                     const double *mb64, cudaStream_t st) {
-    return eval_points32_at(pt_items.ptr, n_items, pt_xy.ptr, pt_perm.ptr, out, sb64, mb64, st);
-}
-
 cudaError_t Fmm::Impl::eval_points32_at(const Tile *items, int n_items, const double *q64, const int *perm,
                                         double *out, const double *sb64, const double *mb64, cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;

@@ -131,12 +131,7 @@ struct Fmm::Impl {
     DevBuf<int> nt_leaves, nt_start, nt_count, nt_perm, nt_own1, nt_own2;
     DevBuf<double> nt_xy;
     int n_nt_leaves = 0;
-    // point targets (eval_points)
-    DevBuf<int> pt_leaves, pt_start, pt_count, pt_perm;
-    DevBuf<double> pt_xy, pt_out;
-    DevBuf<float2> pt_q32;
-    DevBuf<Tile> pt_items;
-    DevBuf<int4> nt_items4, pt_items4;   // (leaf, first target, count, list-1 pieces) work items
+    DevBuf<int4> nt_items4;   // (leaf, first target, count, list-1 pieces) work items
     int n_nt_items4 = 0;
     // near-field coefficients of the node operator (formed once per drawing):
     // single and double layer in FP64, single layer in FP32
@@ -320,11 +315,10 @@ struct Fmm::Impl {
     cudaError_t render_tiles32(int n_tiles, void *rgb, int rgb_dtype,
                                unsigned char *rgb8, const double *sb64, const double *mb64,
                                cudaStream_t st);
-    cudaError_t eval_points32(int n_items, double *out, const double *sb64, const double *mb64,
-                              cudaStream_t st);
     cudaError_t eval_points32_at(const Tile *items, int n_items, const double *q64, const int *perm,
                                  double *out, const double *sb64, const double *mb64, cudaStream_t st);
     PointSort psort;
+    int n_pt_items = 0;           // work items of the sorted points
     evalnodes::NodeArgs<double> node_args64(const int4 *items, const double *q64, const int *own1,
                                             const int *own2, const int *perm, const double *sb,
                                             const double *mb, int use_s, int use_m, double *out) const;
