@@ -13,7 +13,9 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
+#include <utility>
 
 #include "dc_internal.h"
 #include "mlp_tc.cuh"
@@ -22,13 +24,6 @@ namespace dc {
 namespace mlp {
 
 constexpr int kLayers = 4;
-
-__device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float x) {
-    // d/dx [x Phi(x)] = Phi(x) + x phi(x)
-    const float phi = 0.39894228040143268f * __expf(-0.5f * x * x);
-    return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * phi;
-}
 
 __global__ void to_bf16_kernel(const float *__restrict__ a, __nv_bfloat16 *__restrict__ b, size_t n) {
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -54,28 +49,19 @@ __global__ void mse_kernel(const float *__restrict__ Y, const float *__restrict_
     if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
 }
 
+// the loss from the blocks' partial sums, in a fixed order (one warp walking
+// them in turn took 24 us for the 256 of 4,096 rows)
 __global__ void sum_kernel(const float *__restrict__ partial, int n, float scale, float *__restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < n; ++i) s += partial[i];
-        *out = (float)(s * scale);
+    __shared__ double red[256];
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += 256) s += partial[i];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
     }
-}
-
-// dZ = dY * gelu'(Zpre)
-__global__ void gelu_back_kernel(const float *__restrict__ dY, const float *__restrict__ Z,
-                                 float *__restrict__ dZ, size_t n) {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dZ[i] = dY[i] * gelu_grad(Z[i]);
-}
-
-// db[j] = sum_m dZ[m][j], fixed order over m
-__global__ void colsum_kernel(const float *__restrict__ dZ, int M, int N, float *__restrict__ db) {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= N) return;
-    float s = 0.f;
-    for (int m = 0; m < M; ++m) s += dZ[(size_t)m * N + j];
-    db[j] = s;
+    if (threadIdx.x == 0) *out = (float)(red[0] * scale);
 }
 
 __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
@@ -126,27 +112,29 @@ size_t workspace_floats(const Dims &D, int batch) {
     return w;
 }
 
-// C[M][N] = op(A) op(B) (+ bias[N]) (GELU if act), FP32 accumulate.
-//   opA = A [M][K] (lda) or, with ta, A^T of A [K][M]
-//   opB = B^T of B [N][K] (ldb) or, with tb, B [K][N]
-// B may be BF16 (weights) or FP32 (activations).
-void gemm(cudaStream_t st, int M, int N, int K, const float *A, int lda, int ta, const void *B, int ldb,
-          int tb, bool b_bf16, float *C, int ldc, const float *bias, int act, float *Zpre, int *err) {
-    static bool attr = false;
+bool aligned(const void *p, size_t ld_bytes, size_t to) {
+    return (reinterpret_cast<uintptr_t>(p) % to) == 0 && ld_bytes % to == 0;
+}
+
+// C[M][N] = op(A) op(B) with the epilogue of g, FP32 accumulate.
+//   op(A) = A [M][K] or, with TA, A^T of A [K][M]; op(B) = B^T of B [N][K]
+//   or, with TBt, B [K][N], BF16 (weights) or FP32
+template <bool TA, bool TBt, typename TB, int NT, int KC, int NTHR>
+void gemm(cudaStream_t st, GemmArgs g) {
+    auto kernel = gemm_tc_kernel<TA, TBt, TB, NT, KC, NTHR>;
+    constexpr size_t smem = gt_smem(NT, KC);
+    static bool attr = false;   // idempotent: a race sets it twice
     if (!attr) {
-        cudaFuncSetAttribute(gemm_tc_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kGtSmem);
-        cudaFuncSetAttribute(gemm_tc_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGtSmem);
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         attr = true;
     }
-    dim3 grid((M + kGtM - 1) / kGtM, (N + kGtN - 1) / kGtN);
-    if (b_bf16)
-        gemm_tc_kernel<__nv_bfloat16><<<grid, 128, kGtSmem, st>>>(M, N, K, A, lda, ta,
-                                                                 static_cast<const __nv_bfloat16 *>(B), ldb, tb,
-                                                                 C, ldc, bias, act, Zpre, err);
-    else
-        gemm_tc_kernel<float><<<grid, 128, kGtSmem, st>>>(M, N, K, A, lda, ta, static_cast<const float *>(B), ldb,
-                                                         tb, C, ldc, bias, act, Zpre, err);
+    g.veca = aligned(g.A, sizeof(float) * (size_t)g.lda, 16);
+    g.vecb = aligned(g.B, sizeof(TB) * (size_t)g.ldb, 4 * sizeof(TB));
+    g.small = sizeof(float) * (size_t)(TA ? g.K : g.M) * g.lda < (1ull << 32) &&
+              sizeof(TB) * (size_t)(TBt ? g.K : g.N) * g.ldb < (1ull << 32);
+    const size_t ldc = sizeof(float) * (size_t)g.ldc;
+    g.vecc = aligned(g.C, ldc, 16) && aligned(g.Zpre, ldc, 16) && aligned(g.Zback, ldc, 16);
+    kernel<<<dim3((g.M + kGtM - 1) / kGtM, (g.N + NT - 1) / NT), NTHR, smem, st>>>(g);
     note_launch();
 }
 
@@ -192,8 +180,9 @@ dc_status check_waits(const Layout &L, cudaStream_t st) {
     return flag ? DC_ERR_TIMEOUT : DC_OK;
 }
 
-// forward; the output of the last layer is L.Y[3] (linear)
-void forward(const Dims &D, const float *params, int batch, const float *x, const Layout &L,
+// forward into out (the last layer is linear); keep: the pre-activations
+// stay in L.Z for the backward pass
+void forward(const Dims &D, const float *params, int batch, const float *x, const Layout &L, float *out, bool keep,
              cudaStream_t st) {
     size_t n = D.total;
     cudaMemsetAsync(L.err, 0, sizeof(int), st);
@@ -201,9 +190,18 @@ void forward(const Dims &D, const float *params, int batch, const float *x, cons
     dc::note_launch();
     const float *in = x;
     for (int l = 0; l < kLayers; ++l) {
-        const int out = D.d[l + 1], inn = D.d[l];
-        gemm(st, batch, out, inn, in, inn, 0, L.wbf + D.woff[l], inn, 0, true, L.Y[l], out,
-             params + D.boff[l], l + 1 < kLayers ? 1 : 0, L.Z[l], L.err);
+        GemmArgs g{};
+        g.M = batch;
+        g.N = g.ldc = D.d[l + 1];
+        g.K = g.lda = g.ldb = D.d[l];
+        g.A = in;
+        g.B = L.wbf + D.woff[l];
+        g.C = l + 1 < kLayers ? L.Y[l] : out;
+        g.bias = params + D.boff[l];
+        g.act = l + 1 < kLayers;
+        g.Zpre = keep && l + 1 < kLayers ? L.Z[l] : nullptr;
+        g.err = L.err;
+        gemm<false, false, __nv_bfloat16, 64, 1, 256>(st, g);
         in = L.Y[l];
     }
 }
@@ -225,11 +223,8 @@ dc_status dc_aux_mlp_forward(int n_in, int hidden, int n_out, const float *param
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     Dims D = dims(n_in, hidden, n_out);
     Layout L = carve(D, batch, work);
-    forward(D, params, batch, x, L, st);
-    cudaError_t e = cudaMemcpyAsync(y, L.Y[kLayers - 1], sizeof(float) * (size_t)batch * n_out,
-                                    cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) return DC_ERR_CUDA;
+    forward(D, params, batch, x, L, y, false, st);
+    if (cudaGetLastError() != cudaSuccess) return DC_ERR_CUDA;
     return check_waits(L, st);
 }
 
@@ -242,37 +237,44 @@ dc_status dc_aux_mlp_loss_grad(int n_in, int hidden, int n_out, const float *par
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     Dims D = dims(n_in, hidden, n_out);
     Layout L = carve(D, batch, work);
-    forward(D, params, batch, x, L, st);
+    forward(D, params, batch, x, L, L.Y[kLayers - 1], true, st);
     // loss = mean over batch and outputs of (y - t)^2
     size_t ny = (size_t)batch * n_out;
     int nb = (int)((ny + 255) / 256);
     float scale = 1.f / (float)ny;
     mse_kernel<<<nb, 256, 0, st>>>(L.Y[kLayers - 1], target, L.g0, ny, scale, L.partial);
     dc::note_launch();
-    sum_kernel<<<1, 32, 0, st>>>(L.partial, nb, scale, loss);
+    sum_kernel<<<1, 256, 0, st>>>(L.partial, nb, scale, loss);
     dc::note_launch();
-    // backward: g0 holds dL/d(output of layer l) (pre-activation for the last)
+    // backward: dcur holds dL/dZ of layer l; the products of the layer below
+    // are multiplied by gelu' as they leave the accumulator
     float *dcur = L.g0, *dnext = L.g1;
     for (int l = kLayers - 1; l >= 0; --l) {
         const int out = D.d[l + 1], inn = D.d[l];
-        if (l + 1 < kLayers) {
-            size_t n = (size_t)batch * out;
-            gelu_back_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(dcur, L.Z[l], dcur, n);
-            dc::note_launch();
-        }
-        const float *xin = (l == 0) ? x : L.Y[l - 1];
-        // dW [out][inn] = dZ^T [out][batch] x X [batch][inn]
-        gemm(st, out, inn, batch, dcur, out, 1, xin, inn, 1, false, grad + D.woff[l], inn, nullptr, 0,
-             nullptr, L.err);
-        colsum_kernel<<<(out + 127) / 128, 128, 0, st>>>(dcur, batch, out, grad + D.boff[l]);
-        dc::note_launch();
+        // dW [out][inn] = dZ^T [out][batch] x X [batch][inn], db = column sums of dZ
+        GemmArgs g{};
+        g.M = g.lda = out;
+        g.N = g.ldb = g.ldc = inn;
+        g.K = batch;
+        g.A = dcur;
+        g.B = (l == 0) ? x : L.Y[l - 1];
+        g.C = grad + D.woff[l];
+        g.colsum = grad + D.boff[l];
+        g.err = L.err;
+        gemm<true, true, float, 16, 2, 512>(st, g);
         if (l > 0) {
-            // dX [batch][inn] = dZ [batch][out] x W [out][inn]
-            gemm(st, batch, inn, out, dcur, out, 0, L.wbf + D.woff[l], inn, 1, true, dnext, inn, nullptr,
-                 0, nullptr, L.err);
-            float *t = dcur;
-            dcur = dnext;
-            dnext = t;
+            // dX [batch][inn] = dZ [batch][out] x W [out][inn], times gelu'(Z) of the layer below
+            GemmArgs h{};
+            h.M = batch;
+            h.N = h.ldb = h.ldc = inn;
+            h.K = h.lda = out;
+            h.A = dcur;
+            h.B = L.wbf + D.woff[l];
+            h.C = dnext;
+            h.Zback = L.Z[l - 1];
+            h.err = L.err;
+            gemm<false, true, __nv_bfloat16, 64, 1, 256>(st, h);
+            std::swap(dcur, dnext);
         }
     }
     if (cudaGetLastError() != cudaSuccess) return DC_ERR_CUDA;
