@@ -1,0 +1,94 @@
+// Targets evaluated in float-float (ffmath.cuh): the pixels of the FP64 FMM
+// form and of the dense form.  Segments are staged in shared memory in a
+// frame around the targets, differences taken in FP64 (once per segment and
+// block), then held as (hi, lo) floats.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "ffmath.cuh"
+
+namespace dc {
+namespace evalff {
+
+constexpr int kStage = 64;   // segments staged per round
+
+struct Stage {
+    // x1 y1 | x2 y2 | dx dy, each (hi, lo); len and the weights of the three
+    // channels: -w sigma / 2 pi and -w mu / 2 pi
+    float4 p1[kStage], p2[kStage], d[kStage];
+    float2 len[kStage], sg[kStage][3], mg[kStage][3];
+};
+
+// Entry i of the stage: the segment q (x1 y1 x2 y2) relative to (cx, cy),
+// times iw (a power of two); ks, km: what multiplies sb and mb.
+__device__ __forceinline__ void stage_segment(Stage &t, int i, const double *__restrict__ q, double cx, double cy,
+                                              float iw, double len, double ks, double km,
+                                              const double *__restrict__ sb, const double *__restrict__ mb) {
+    const float2 x1 = ff::scale(ff::from(q[0] - cx), iw), y1 = ff::scale(ff::from(q[1] - cy), iw);
+    const float2 x2 = ff::scale(ff::from(q[2] - cx), iw), y2 = ff::scale(ff::from(q[3] - cy), iw);
+    const float2 dx = ff::scale(ff::from(q[2] - q[0]), iw), dy = ff::scale(ff::from(q[3] - q[1]), iw);
+    t.p1[i] = make_float4(x1.x, x1.y, y1.x, y1.y);
+    t.p2[i] = make_float4(x2.x, x2.y, y2.x, y2.y);
+    t.d[i] = make_float4(dx.x, dx.y, dy.x, dy.y);
+    t.len[i] = ff::scale(ff::from(len), iw);
+    for (int c = 0; c < 3; ++c) {
+        t.sg[i][c] = ff::from(ks * sb[c]);
+        t.mg[i][c] = ff::from(km * mb[c]);
+    }
+}
+
+// A sum of three channels: a short run in float-float (hi, lo), flushed into
+// FP64 round by round.  The lo parts of a long run would lose what they hold:
+// 5,120 large, cancelling terms summed without a flush were 1e-11 off, the
+// pairs themselves 4e-15.
+struct Sum3 {
+    float h[3], l[3];
+    double v[3];
+    __device__ __forceinline__ void zero() {
+        for (int c = 0; c < 3; ++c) {
+            h[c] = l[c] = 0.f;
+            v[c] = 0.0;
+        }
+    }
+    __device__ __forceinline__ void flush() {
+        for (int c = 0; c < 3; ++c) {
+            v[c] += (double)h[c] + l[c];
+            h[c] = l[c] = 0.f;
+        }
+    }
+};
+// u += entry i's single and double layer at the target (x, y) of the frame
+__device__ __forceinline__ void add_segment(const ff::Tables &T, const Stage &t, int i, float2 x, float2 y, Sum3 &u) {
+    const float4 p1 = t.p1[i], p2 = t.p2[i], d = t.d[i];
+    float2 il, ph;
+    ff::pair(T, ff::sub(make_float2(p1.x, p1.y), x), ff::sub(make_float2(p1.z, p1.w), y),
+             ff::sub(make_float2(p2.x, p2.y), x), ff::sub(make_float2(p2.z, p2.w), y), make_float2(d.x, d.y),
+             make_float2(d.z, d.w), t.len[i], il, ph);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        dot2ff(u.h[c], u.l[c], il, t.sg[i][c]);
+        dot2ff(u.h[c], u.l[c], ph, t.mg[i][c]);
+    }
+}
+
+// u += Re sum_k C[c][k] p^k, k = 0 .. n - 1, for complex (px, py) and
+// coefficients (re hi, re lo, im hi, im lo); the powers are shared by the
+// three channels
+__device__ __forceinline__ void add_powers(const float4 *__restrict__ C, int stride, int n, float2 px, float2 py, Sum3 &u) {
+    float2 wx = make_float2(1.f, 0.f), wy = make_float2(0.f, 0.f);
+    for (int k = 0; k < n; ++k) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float4 v = C[c * stride + k];
+            dot2ff(u.h[c], u.l[c], make_float2(v.x, v.y), wx);
+            dot2ff(u.h[c], u.l[c], make_float2(-v.z, -v.w), wy);
+        }
+        const float2 t = ff::dot(wx, px, ff::neg(wy), py);
+        wy = ff::dot(wx, py, wy, px);
+        wx = t;
+    }
+}
+
+}  // namespace evalff
+}  // namespace dc

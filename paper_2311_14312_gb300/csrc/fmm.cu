@@ -37,6 +37,7 @@
 #include "fmm_impl.h"
 #include "passes.cuh"
 #include "passes_tc.cuh"
+#include "evalff.cuh"
 #include "segint.cuh"
 
 namespace dc {
@@ -49,157 +50,137 @@ namespace {
 
 using cd = std::complex<double>;
 
-// ----------------------------------------------------- complex helpers --
-__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ double2 cadd(double2 a, double2 b) {
-    return make_double2(a.x + b.x, a.y + b.y);
-}
-__device__ __forceinline__ double2 cscale(double2 a, double s) {
-    return make_double2(a.x * s, a.y * s);
-}
-__device__ __forceinline__ double2 cinv(double2 a) {
-    double d = 1.0 / (a.x * a.x + a.y * a.y);
-    return make_double2(a.x * d, -a.y * d);
-}
-// principal log
-__device__ __forceinline__ double2 clog(double2 a) {
-    return make_double2(0.5 * log(a.x * a.x + a.y * a.y), atan2(a.y, a.x));
-}
-// acc += m * v (complex)
-__device__ __forceinline__ void cfma(double2 &acc, double2 m, double2 v) {
-    acc.x += m.x * v.x - m.y * v.y;
-    acc.y += m.x * v.y + m.y * v.x;
-}
-
-
-
 // ------------------------------------------------------------- eval ----
-struct Acc3 {
-    double v[3];
-};
-
-__device__ __forceinline__ void eval_point(const DevTree &t, int leaf, double qx, double qy,
-                                           int own1, int own2, int P1,
-                                           const double2 *__restrict__ M,
-                                           const double2 *__restrict__ L,
-                                           const double *__restrict__ sbar,
-                                           const double *__restrict__ mbar, int use_s, int use_m,
-                                           Acc3 &u, long long &pairs) {
-    double e0 = 0, e1 = 0, e2 = 0;   // expansion parts, times 2 pi
-    // L2P (Eq. 64)
-    {
-        double w = t.cw[leaf];
-        double2 z = make_double2((qx - t.cc[2 * leaf]) / w, (qy - t.cc[2 * leaf + 1]) / w);
-        const double2 *Lc = L + (size_t)leaf * 3 * P1;
-        double2 s0 = Lc[P1 - 1], s1 = Lc[2 * P1 - 1], s2 = Lc[3 * P1 - 1];
-        for (int k = P1 - 2; k >= 0; --k) {
-            s0 = cadd(cmul(s0, z), Lc[k]);
-            s1 = cadd(cmul(s1, z), Lc[P1 + k]);
-            s2 = cadd(cmul(s2, z), Lc[2 * P1 + k]);
-        }
-        e0 += s0.x;
-        e1 += s1.x;
-        e2 += s2.x;
-    }
-    // M2P over list 3 (Eq. 61)
-    for (int e = t.w_ptr[leaf]; e < t.w_ptr[leaf + 1]; ++e) {
-        int src = t.w_idx[e];
-        double w = t.cw[src];
-        double zx = qx - t.cc[2 * src], zy = qy - t.cc[2 * src + 1];
-        double2 iz = cinv(make_double2(zx / w, zy / w));
-        double lz = 0.5 * log(zx * zx + zy * zy);
-        const double2 *Ms = M + (size_t)src * 3 * P1;
-        double2 s[3];
-        for (int c = 0; c < 3; ++c) s[c] = cscale(Ms[c * P1 + P1 - 1], 1.0 / (P1 - 1));
-        for (int k = P1 - 2; k >= 1; --k)
-            for (int c = 0; c < 3; ++c) s[c] = cadd(cmul(s[c], iz), cscale(Ms[c * P1 + k], 1.0 / k));
-        for (int c = 0; c < 3; ++c) s[c] = cmul(s[c], iz);
-        e0 += s[0].x - lz * Ms[0].x;
-        e1 += s[1].x - lz * Ms[P1].x;
-        e2 += s[2].x - lz * Ms[2 * P1].x;
-    }
-    double u0 = e0 * kInv2Pi, u1 = e1 * kInv2Pi, u2 = e2 * kInv2Pi;
-    // P2P over list 1 (App. D closed forms)
-    for (int e = t.u_ptr[leaf]; e < t.u_ptr[leaf + 1]; ++e) {
-        int src = t.u_idx[e];
-        int p0 = t.pstart[src], pn = t.pcount[src];
-        pairs += pn;
-        for (int i = p0; i < p0 + pn; ++i) {
-            const double *q = t.pc + 4 * (size_t)i;
-            int seg = t.pseg[i];
-            double G, F;
-            seg_gf_f64(qx, qy, q[0], q[1], q[2], q[3], t.pw[i], seg == own1 || seg == own2, G, F);
-            if (use_s) {
-                u0 += G * sbar[3 * (size_t)seg + 0];
-                u1 += G * sbar[3 * (size_t)seg + 1];
-                u2 += G * sbar[3 * (size_t)seg + 2];
-            }
-            if (use_m) {
-                u0 += F * mbar[3 * (size_t)seg + 0];
-                u1 += F * mbar[3 * (size_t)seg + 1];
-                u2 += F * mbar[3 * (size_t)seg + 2];
-            }
-        }
-    }
-    u.v[0] = u0;
-    u.v[1] = u1;
-    u.v[2] = u2;
-}
-
-// Targets grouped by leaf (nodes or sorted points); result scattered to the
-// original order.
-__global__ void eval_targets_kernel(DevTree t, const int *__restrict__ leaves,
-                                    const int *__restrict__ tstart, const int *__restrict__ tcount,
-                                    const double *__restrict__ txy, const int *__restrict__ town1,
-                                    const int *__restrict__ town2, const int *__restrict__ tperm,
-                                    int P1, const double2 *__restrict__ M,
-                                    const double2 *__restrict__ L, const double *__restrict__ sbar,
-                                    const double *__restrict__ mbar, int use_s, int use_m,
-                                    double *__restrict__ out) {
-    int leaf = leaves[blockIdx.x];
-    int s0 = tstart[leaf], n = tcount[leaf];
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        int ti = s0 + j;
-        Acc3 u;
-        long long pairs = 0;
-        eval_point(t, leaf, txy[2 * ti], txy[2 * ti + 1], town1 ? town1[ti] : -1,
-                   town2 ? town2[ti] : -1, P1, M, L, sbar, mbar, use_s, use_m, u, pairs);
-        int o = tperm[ti];
-        out[3 * (size_t)o + 0] = u.v[0];
-        out[3 * (size_t)o + 1] = u.v[1];
-        out[3 * (size_t)o + 2] = u.v[2];
-    }
-}
-
-
-
 __device__ __forceinline__ unsigned char q8(double v) {
     v = fmin(fmax(v, 0.0), 1.0);
     return (unsigned char)floor(255.0 * v + 0.5);
 }
 
-__global__ void eval_tiles_kernel(DevTree t, const RTile *__restrict__ tiles, const VpDev *__restrict__ vps, int P1,
-                                  const double2 *__restrict__ M, const double2 *__restrict__ L,
-                                  const double *__restrict__ sbar, const double *__restrict__ mbar,
-                                  void *rgb, int rgb_dtype, unsigned char *rgb8) {
-    const RTile tl = tiles[blockIdx.x];
-    const VpDev vp = vps[tl.vp];
-    int npx = tl.nr * tl.nc;
-    for (int j = threadIdx.x; j < npx; j += blockDim.x) {
-        int r = tl.r0 + j / tl.nc, c = tl.c0 + j % tl.nc;
-        double qx = vp.x0 + (c + 0.5) * vp.dx, qy = vp.y0 + (r + 0.5) * vp.dy;
-        Acc3 u;
-        long long pairs = 0;
-        eval_point(t, tl.leaf, qx, qy, -1, -1, P1, M, L, sbar, mbar, 1, 1, u, pairs);
-        size_t o = 3 * ((size_t)vp.offset + (size_t)r * vp.width + c);
-        for (int ch = 0; ch < 3; ++ch) {
-            if (rgb) {
-                if (rgb_dtype == DC_F64) static_cast<double *>(rgb)[o + ch] = u.v[ch];
-                else static_cast<float *>(rgb)[o + ch] = (float)u.v[ch];
+// The FP64 form's pixels in float-float: a block of 64 threads takes
+// rectangles of up to 8 x 8 pixels of one leaf from the counter, one pixel a
+// thread, in the leaf's frame (origin its centre, its width scaled to one: a
+// power of two; the logarithms are then log(r / w), and the constant rest,
+// log(w) times the pieces' total weighted length, is added in FP64).  Bound by
+// FP32 issue: 450 instructions a pair and 100 a coefficient and channel
+// triple.  517 x 509 pixels of a 48-curve drawing (76 list-1 pieces and 7
+// list-3 cells a pixel) in 1.12 ms on one GB300, 9.95 with the pairs and
+// expansions in FP64, whose pipe they saturated; the error against a 64-bit
+// direct sum is the same 1.6e-12 (the expansions' truncation).
+constexpr int kFfThreads = 64, kFfBlocksPerSM = 8;
+__global__ void __launch_bounds__(kFfThreads, kFfBlocksPerSM)
+eval_tiles_kernel(DevTree t, const RTile *__restrict__ tiles, int n_tiles, int *__restrict__ queue,
+                  const VpDev *__restrict__ vps, int P1, const double *__restrict__ plen,
+                  const int *__restrict__ uf_ptr, const int *__restrict__ uf_idx, const double2 *__restrict__ M,
+                  const double2 *__restrict__ L, const double *__restrict__ sbar, const double *__restrict__ mbar,
+                  void *rgb, int rgb_dtype, unsigned char *rgb8) {
+    __shared__ ff::Tables T;
+    __shared__ evalff::Stage S;
+    __shared__ float4 coef[3 * (kMaxP + 1)];
+    __shared__ double red[kFfThreads / 32][3];
+    __shared__ int next;
+    ff::init_tables(T);
+    while (true) {
+        __syncthreads();
+        if (threadIdx.x == 0) next = atomicAdd(queue, 1);
+        __syncthreads();
+        if (next >= n_tiles) break;
+        const RTile tl = tiles[next];
+        const VpDev &vp = vps[tl.vp];
+        const int leaf = tl.leaf, npx = tl.nr * tl.nc, j = threadIdx.x;
+        const double cx = t.cc[2 * leaf], cy = t.cc[2 * leaf + 1], w = t.cw[leaf];
+        const float iw = (float)(1.0 / w);   // exact: a power of two
+        const bool on = j < npx;
+        const int r = tl.r0 + (on ? j / tl.nc : 0), c = tl.c0 + (on ? j % tl.nc : 0);
+        const float2 x = ff::scale(ff::from(vp.x0 + (c + 0.5) * vp.dx - cx), iw);
+        const float2 y = ff::scale(ff::from(vp.y0 + (r + 0.5) * vp.dy - cy), iw);
+        evalff::Sum3 u, e;   // list 1; expansions, times 2 pi
+        u.zero();
+        e.zero();
+        // L2P (Eq. 64)
+        for (int i = j; i < 3 * P1; i += kFfThreads) {
+            const double2 v = L[(size_t)leaf * 3 * P1 + i];
+            const float2 a = ff::from(v.x), b = ff::from(v.y);
+            coef[i] = make_float4(a.x, a.y, b.x, b.y);
+        }
+        __syncthreads();
+        evalff::add_powers(coef, P1, P1, x, y, e);
+        e.flush();
+        // M2P over list 3 (Eq. 61): sum_k M_k / k z^-k - log|z| M_0, z in the cell's widths
+        for (int k = t.w_ptr[leaf]; k < t.w_ptr[leaf + 1]; ++k) {
+            const int src = t.w_idx[k];
+            const double ws = t.cw[src];
+            __syncthreads();
+            for (int i = j; i < 3 * P1; i += kFfThreads) {
+                const int q = i % P1;
+                double2 v = M[(size_t)src * 3 * P1 + i];
+                if (q > 1) {
+                    const double iq = 1.0 / q;
+                    v.x *= iq;
+                    v.y *= iq;
+                }
+                const float2 a = ff::from(v.x), b = ff::from(v.y);
+                coef[i] = make_float4(a.x, a.y, b.x, b.y);
             }
-            if (rgb8) rgb8[o + ch] = q8(u.v[ch]);
+            __syncthreads();
+            const float rw = (float)(w / ws);   // a power of two
+            const float2 ox = ff::from((cx - t.cc[2 * src]) / ws), oy = ff::from((cy - t.cc[2 * src + 1]) / ws);
+            const float2 zx = ff::add(ff::scale(x, rw), ox), zy = ff::add(ff::scale(y, rw), oy);
+            const float2 r2 = ff::dot(zx, zx, zy, zy), ir = ff::inv(r2);
+            const float2 lz = ff::neg(ff::add(ff::scale(ff::log(T, r2), 0.5f), ff::from(log(ws))));
+            const float2 px = ff::mul(zx, ir), py = ff::neg(ff::mul(zy, ir));
+            for (int ch = 0; ch < 3; ++ch) {
+                const float4 m0 = coef[ch * P1];
+                dot2ff(e.h[ch], e.l[ch], make_float2(m0.x, m0.y), lz);
+            }
+            // k >= 1: the powers from z^-1 on
+            float2 wx = px, wy = py;
+            for (int q = 1; q < P1; ++q) {
+#pragma unroll
+                for (int ch = 0; ch < 3; ++ch) {
+                    const float4 v = coef[ch * P1 + q];
+                    dot2ff(e.h[ch], e.l[ch], make_float2(v.x, v.y), wx);
+                    dot2ff(e.h[ch], e.l[ch], make_float2(-v.z, -v.w), wy);
+                }
+                const float2 s = ff::dot(wx, px, ff::neg(wy), py);
+                wy = ff::dot(wx, py, wy, px);
+                wx = s;
+            }
+            e.flush();
+        }
+        // P2P over list 1 (App. D closed forms)
+        double k3[3] = {0.0, 0.0, 0.0};   // weighted lengths of the pieces this thread staged
+        for (int f0 = uf_ptr[leaf]; f0 < uf_ptr[leaf + 1]; f0 += evalff::kStage) {
+            const int n = min(evalff::kStage, uf_ptr[leaf + 1] - f0);
+            __syncthreads();
+            if (j < n) {
+                const int i = uf_idx[f0 + j];
+                const size_t s3 = 3 * (size_t)t.pseg[i];
+                const double wg = -t.pw[i] * kInv2Pi, len = plen[i];
+                evalff::stage_segment(S, j, t.pc + 4 * (size_t)i, cx, cy, iw, len, wg * w, wg, sbar + s3, mbar + s3);
+                for (int ch = 0; ch < 3; ++ch) k3[ch] += wg * len * sbar[s3 + ch];
+            }
+            __syncthreads();
+            if (on)
+                for (int i = 0; i < n; ++i) evalff::add_segment(T, S, i, x, y, u);
+            u.flush();
+        }
+        for (int ch = 0; ch < 3; ++ch) {
+            for (int o = 16; o > 0; o >>= 1) k3[ch] += __shfl_xor_sync(0xffffffffu, k3[ch], o);
+            if ((j & 31) == 0) red[j >> 5][ch] = k3[ch];
+        }
+        __syncthreads();
+        if (on) {
+            const double lw = log(w);
+            const size_t o = 3 * ((size_t)vp.offset + (size_t)r * vp.width + c);
+            for (int ch = 0; ch < 3; ++ch) {
+                const double v = u.v[ch] + e.v[ch] * kInv2Pi +
+                                 (red[0][ch] + red[1][ch]) * lw;
+                if (rgb) {
+                    if (rgb_dtype == DC_F64) static_cast<double *>(rgb)[o + ch] = v;
+                    else static_cast<float *>(rgb)[o + ch] = (float)v;
+                }
+                if (rgb8) rgb8[o + ch] = q8(v);
+            }
         }
     }
 }
@@ -1704,9 +1685,15 @@ static dc_status launch_render(Fmm::Impl &I, int n_tiles, void *rgb, int rgb_dty
     if (I.fp32)
         e = I.render_tiles32(n_tiles, rgb, rgb_dtype, rgb8, sbar, mbar, st);
     else {
-        eval_tiles_kernel<<<n_tiles, 128, 0, st>>>(I.dt(), I.tiles.ptr, I.vps.ptr, I.P1,
-                                                              I.M.ptr, I.L.ptr, sbar, mbar, rgb,
-                                                              rgb_dtype, rgb8);
+        if ((e = I.render_queue.ensure(1)) == cudaSuccess)
+            e = cudaMemsetAsync(I.render_queue.ptr, 0, sizeof(int), st);
+        if (e != cudaSuccess) {
+            err = cudaGetErrorString(e);
+            return e == cudaErrorMemoryAllocation ? DC_ERR_OOM : DC_ERR_CUDA;
+        }
+        eval_tiles_kernel<<<std::min(n_tiles, I.n_sms * kFfBlocksPerSM), kFfThreads, 0, st>>>(
+            I.dt(), I.tiles.ptr, n_tiles, I.render_queue.ptr, I.vps.ptr, I.P1, I.plen64.ptr, I.uf_ptr.ptr, I.uf_idx.ptr,
+            I.M.ptr, I.L.ptr, sbar, mbar, rgb, rgb_dtype, rgb8);
         note_launch();
         e = cudaGetLastError();
     }
