@@ -70,8 +70,8 @@ constexpr int kFfThreads = 64, kFfBlocksPerSM = 8;
 __global__ void __launch_bounds__(kFfThreads, kFfBlocksPerSM)
 eval_tiles_kernel(DevTree t, const RTile *__restrict__ tiles, int n_tiles, int *__restrict__ queue,
                   const VpDev *__restrict__ vps, int P1, const double *__restrict__ plen,
-                  const int *__restrict__ uf_ptr, const int *__restrict__ uf_idx, const double2 *__restrict__ M,
-                  const double2 *__restrict__ L, const double *__restrict__ sbar, const double *__restrict__ mbar,
+                  const int *__restrict__ uf_ptr, const int *__restrict__ uf_idx, const float4 *__restrict__ M,
+                  const float4 *__restrict__ L, const double *__restrict__ sbar, const double *__restrict__ mbar,
                   void *rgb, int rgb_dtype, unsigned char *rgb8) {
     __shared__ ff::Tables T;
     __shared__ evalff::Stage S;
@@ -98,9 +98,8 @@ eval_tiles_kernel(DevTree t, const RTile *__restrict__ tiles, int n_tiles, int *
         e.zero();
         // L2P (Eq. 64)
         for (int i = j; i < 3 * P1; i += kFfThreads) {
-            const double2 v = L[(size_t)leaf * 3 * P1 + i];
-            const float2 a = ff::from(v.x), b = ff::from(v.y);
-            coef[i] = make_float4(a.x, a.y, b.x, b.y);
+            const float4 v = L[(size_t)leaf * 3 * P1 + i];   // re hi, im hi, re lo, im lo
+            coef[i] = make_float4(v.x, v.z, v.y, v.w);
         }
         __syncthreads();
         evalff::add_powers(coef, P1, P1, x, y, e);
@@ -112,13 +111,13 @@ eval_tiles_kernel(DevTree t, const RTile *__restrict__ tiles, int n_tiles, int *
             __syncthreads();
             for (int i = j; i < 3 * P1; i += kFfThreads) {
                 const int q = i % P1;
-                double2 v = M[(size_t)src * 3 * P1 + i];
+                const float4 v = M[(size_t)src * 3 * P1 + i];
+                float2 a = make_float2(v.x, v.z), b = make_float2(v.y, v.w);
                 if (q > 1) {
-                    const double iq = 1.0 / q;
-                    v.x *= iq;
-                    v.y *= iq;
+                    const float2 iq = ff::inv(make_float2((float)q, 0.f));
+                    a = ff::mul(a, iq);
+                    b = ff::mul(b, iq);
                 }
-                const float2 a = ff::from(v.x), b = ff::from(v.y);
                 coef[i] = make_float4(a.x, a.y, b.x, b.y);
             }
             __syncthreads();
@@ -247,6 +246,21 @@ void build_base_tables(int p, std::vector<cd> &base) {
     }
 }
 
+// An M2M (up) or L2L table [4][P1][P1] in the order the lanes of passes.cuh's
+// pair_sums read it: [quadrant][step][lane], zero where a lane has no term.
+std::vector<cd> lane_order(const std::vector<cd> &t, bool up, int P1) {
+    std::vector<cd> o((size_t)4 * (P1 + 1) * passes::kPairLanes, cd(0));
+    for (int q = 0; q < 4; ++q)
+        for (int i = 0; i <= P1; ++i)
+            for (int kk = 0; 2 * kk < P1; ++kk) {
+                const bool second = i >= passes::pair_switch(up, P1, kk);
+                if (second && 2 * kk == P1 - 1) continue;   // the middle lane has one output
+                const int out = second ? P1 - 1 - kk : kk, in = passes::pair_in(up, P1, kk, i);
+                o[((size_t)q * (P1 + 1) + i) * passes::kPairLanes + kk] = t[((size_t)q * P1 + out) * P1 + in];
+            }
+    return o;
+}
+
 // The tables of an expansion order, built once per process and kept (they
 // depend on p alone; entries are never removed, so references stay valid).
 struct OrderTables {
@@ -350,54 +364,78 @@ passes::TreeView<double> Fmm::Impl::view64() const {
 // Up and down passes for segment densities (sbar / mbar), FP64.
 cudaError_t Fmm::Impl::passes(const double *sb, const double *mb, int use_s, int use_m,
                               cudaStream_t st, const Schedule &sc) {
-    const int nC = tree.n_cells();
-    size_t ebytes = (size_t)nC * 3 * P1 * sizeof(double2);
+    const size_t nE = (size_t)tree.n_cells() * 3 * P1;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(M.ptr, 0, ebytes, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(L.ptr, 0, ebytes, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(Lm2l.ptr, 0, ebytes, st)) != cudaSuccess) return e;
     passes::TreeView<double> tv = view64();
     passes::PiecesF64 ps{pc.ptr, cc.ptr};
+    // On the 200-curve drawing (11,529 cells, 13 levels, order 24, one GB300)
+    // all of it takes 0.56 ms, 0.94 with a launch per level and warp per cell
+    // in FP64 storage: upward 229 -> 94 us, downward 204 -> 116 us, list 4
+    // (117 us) out of the way; list 2 (222 us) is bound by FP32 issue.
+    // The list-4 terms need the densities alone: their stored rows stream
+    // from memory beside the latency-bound P2M and upward pass, and the list-2
+    // terms are added onto them.  Cells without list 4 start from zero, and
+    // so does every L (leaves above level 2 have no terms at all).
+    const bool p2l = sc.n_p2l > 0;
+    const cudaStream_t s2 = rows_ready ? p2l_stream : st;
+    if (s2 != st && ((e = cudaEventRecord(p2l_ev[0], st)) != cudaSuccess ||
+                     (e = cudaStreamWaitEvent(s2, p2l_ev[0], 0)) != cudaSuccess))
+        return e;
+    if ((e = cudaMemsetAsync(Lxff.ptr, 0, nE * sizeof(float4), s2)) != cudaSuccess ||
+        (e = cudaMemsetAsync(Lff.ptr, 0, nE * sizeof(float4), s2)) != cudaSuccess)
+        return e;
+    if (p2l && rows_ready) {
+        passes::p2l_rows_ff_kernel<<<sc.n_p2l, passes::kChunk, 0, s2>>>(tv, sc.p2l.ptr, p2l_off.ptr, p2l_cnt.ptr,
+                                                                       p2l_item.ptr, sb, mb, use_s, use_m, P1, Lxff.ptr,
+                                                                       p2l_gff.ptr, p2l_fff.ptr);
+        note_launch();
+    } else if (p2l) {   // the rows would not fit: recomputed in FP64
+        if ((e = cudaMemsetAsync(Lm2l.ptr, 0, nE * sizeof(double2), st)) != cudaSuccess) return e;
+        passes::p2l_kernel<double, passes::PiecesF64><<<sc.n_p2l, passes::kChunk, passes::p2l_smem<double>(P1), st>>>(
+            tv, ps, sc.p2l.ptr, sb, mb, use_s, use_m, P1, Lm2l.ptr);
+        passes::rows_to_ff_kernel<<<4 * n_sms, 256, 0, st>>>(Lm2l.ptr, Lxff.ptr, nE);
+        note_launch(2);
+    }
+    if (s2 != st && (e = cudaEventRecord(p2l_ev[1], s2)) != cudaSuccess) return e;
     if (n_p2m > 0) {
-        if (rows_ready)
+        if (rows_ready) {
             passes::p2m_rows_ff_kernel<<<n_p2m, passes::kChunk, 0, st>>>(tv, p2m_leaves.ptr, sb, mb, use_s, use_m, P1,
-                                                                       M.ptr, p2m_gff.ptr, p2m_fff.ptr);
-        else
+                                                                       Mff.ptr, p2m_gff.ptr, p2m_fff.ptr);
+        } else {
             passes::p2m_kernel<double, passes::PiecesF64><<<n_p2m, passes::kChunk, passes::p2m_smem<double>(P1), st>>>(
                 tv, ps, p2m_leaves.ptr, sb, mb, use_s, use_m, P1, M.ptr);
+            passes::rows_to_ff_kernel<<<4 * n_sms, 256, 0, st>>>(M.ptr, Mff.ptr, nE);   // inner cells follow
+            note_launch();
+        }
         note_launch();
     }
-    // per level, in float-float: the chain through the parents does less
-    // arithmetic than translating every leaf to every ancestor
-    for (int l = tree.depth - 1; l >= 2; --l) {
-        const int lo = m2m_ptr[l], n = m2m_ptr[l + 1] - lo;
-        if (n <= 0) continue;
-        passes::m2m_ff_kernel<<<(n + 3) / 4, 128, passes::mlff_smem(P1), st>>>(child0.ptr, m2m_cells.ptr + lo, n, P1,
-                                                                            m2mff.ptr, M.ptr);
+    if (n_up > 0) {
+        passes::m2m_up_kernel<<<n_up, passes::kPairThreads, 0, st>>>(child0.ptr, parent.ptr, up_starts.ptr, up_need.ptr,
+                                                                    up_arrived.ptr, P1, m2mff.ptr, Mff.ptr);
         note_launch();
     }
+    if (s2 != st && (e = cudaStreamWaitEvent(st, p2l_ev[1], 0)) != cudaSuccess) return e;
     if (sc.n_m2l > 0) {
         int grid = std::min((sc.n_m2l + passes::kM2LffWarps - 1) / passes::kM2LffWarps, 4 * n_sms);
         passes::m2l_ff_kernel<<<grid, 32 * passes::kM2LffWarps, passes::m2l_ff_smem(P1), st>>>(
-            tv, sc.m2l.ptr, sc.n_m2l, P1, baseff.ptr, M.ptr, Lm2l.ptr);
+            tv, sc.m2l.ptr, sc.n_m2l, P1, baseff.ptr, Mff.ptr, Lxff.ptr);
         note_launch();
     }
-    if (sc.n_p2l > 0) {
-        if (rows_ready)
-            passes::p2l_rows_ff_kernel<<<sc.n_p2l, passes::kChunk, 0, st>>>(
-                tv, sc.p2l.ptr, p2l_off.ptr, p2l_cnt.ptr, p2l_item.ptr, sb, mb, use_s, use_m, P1, Lm2l.ptr,
-                p2l_gff.ptr, p2l_fff.ptr);
-        else
-            passes::p2l_kernel<double, passes::PiecesF64><<<sc.n_p2l, passes::kChunk, passes::p2l_smem<double>(P1), st>>>(
-                tv, ps, sc.p2l.ptr, sb, mb, use_s, use_m, P1, Lm2l.ptr);
-        note_launch();
-    }
-    for (int l = 2; l <= tree.depth; ++l) {   // per level: FP64 work per cell once
-        const int lo = sc.l2l_ptr[l], n = sc.l2l_ptr[l + 1] - lo;
+    for (size_t i = 0; i + 1 < sc.l2l_ptr.size(); ++i) {
+        const int lo = sc.l2l_ptr[i], n = sc.l2l_ptr[i + 1] - lo;
         if (n <= 0) continue;
-        passes::l2l_ff_kernel<<<(n + 3) / 4, 128, 0, st>>>(tv, sc.l2l.ptr + lo, n, l, P1, l2lff.ptr, Lm2l.ptr, L.ptr);
+        passes::l2l_two_kernel<<<n, passes::kPairThreads, 0, st>>>(child0.ptr, parent.ptr, quad.ptr, sc.l2l.ptr + lo,
+                                                                  i > 0 ? 1 : 0, P1, l2lff.ptr, Lxff.ptr, Lff.ptr);
         note_launch();
     }
+    return cudaGetLastError();
+}
+
+cudaError_t Fmm::Impl::widen(cudaStream_t st) {
+    const size_t nE = (size_t)tree.n_cells() * 3 * P1;
+    passes::ff_to_rows_kernel<<<4 * n_sms, 256, 0, st>>>(Mff.ptr, M.ptr, nE);
+    passes::ff_to_rows_kernel<<<4 * n_sms, 256, 0, st>>>(Lff.ptr, L.ptr, nE);
+    note_launch(2);
     return cudaGetLastError();
 }
 
@@ -452,6 +490,8 @@ cudaError_t Fmm::Impl::eval_list64(const int4 *items, int n_items, const double 
                                    const double *sb, const double *mb, int use_s, int use_m,
                                    double *out, cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;
+    cudaError_t e = widen(st);
+    if (e != cudaSuccess) return e;
     evalnodes::NodeArgs<double> a = node_args64(items, q64, own1, own2, perm, sb, mb, use_s, use_m, out);
     evalnodes::eval_nodes_kernel<double><<<n_items, 32 * evalnodes::kWarps, 0, st>>>(a);
     note_launch();
@@ -465,22 +505,18 @@ cudaError_t Fmm::Impl::apply_nodes(const double *x, double *y, bool single, cuda
     if ((e = passes(sbar.ptr, mbar.ptr, us, um, st, sched_nodes)) != cudaSuccess) return e;
     if (near_ready && far_ready && n_nt_items4 > 0) {   // float-float from stored coefficients
         const long long nS = 3LL * D->S;
-        const size_t nE = (size_t)tree.n_cells() * 3 * P1;
-        if ((e = dens_ff.ensure((size_t)nS)) != cudaSuccess || (e = Lff.ensure(nE)) != cudaSuccess ||
-            (e = Mff.ensure(nE)) != cudaSuccess)
-            return e;
+        if ((e = dens_ff.ensure((size_t)nS)) != cudaSuccess) return e;
         d2ff_kernel<<<4 * n_sms, 256, 0, st>>>(single ? sbar.ptr : mbar.ptr, dens_ff.ptr, nS);
-        passes::rows_to_ff_kernel<<<4 * n_sms, 256, 0, st>>>(L.ptr, Lff.ptr, nE);
-        passes::rows_to_ff_kernel<<<4 * n_sms, 256, 0, st>>>(M.ptr, Mff.ptr, nE);
         evalnodes::NodeArgs<double> a = node_args64(nt_items4.ptr, nt_xy.ptr, nt_own1.ptr, nt_own2.ptr,
                                                     nt_perm.ptr, sbar.ptr, mbar.ptr, us, um, y);
         evalnodes::near_apply_ff_kernel<<<n_nt_items4, 32 * evalnodes::kWarps, 0, st>>>(
             a, near_off.ptr, single ? near_gff.ptr : near_fff.ptr, dens_ff.ptr, far_off.ptr, farff.ptr, Lff.ptr,
             Mff.ptr);
-        note_launch(4);
+        note_launch(2);
         return cudaGetLastError();
     }
     if (near_ready && n_nt_items4 > 0) {
+        if ((e = widen(st)) != cudaSuccess) return e;
         evalnodes::NodeArgs<double> a = node_args64(nt_items4.ptr, nt_xy.ptr, nt_own1.ptr, nt_own2.ptr,
                                                     nt_perm.ptr, sbar.ptr, mbar.ptr, us, um, y);
         evalnodes::near_apply_kernel<double><<<n_nt_items4, 32 * evalnodes::kWarps, 0, st>>>(
@@ -830,21 +866,26 @@ dc_status Fmm::build(const dc_options &opt, const Geometry &G, const DevGeom &D,
     // pass schedules: inner cells of level >= 2 with pieces, by level; the
     // leaf -> ancestor M2M pairs of every inner cell, chunked for the
     // one-launch upward pass (cells with several chunks get partial slots)
-    std::vector<int> m2m_cells;
+    std::vector<int> m2m_cells, up_starts, up_need;
     std::vector<int4> mchunks, mred;
     std::vector<int> pair_leaf;
     std::vector<float4> pair_geo;
     int n_slots = 0;
     Joiner j_mchunks;
     j_mchunks.run(guarded([&] {
-        I.m2m_ptr.assign(T.depth + 2, 0);
-        for (int l = 0; l <= T.depth; ++l) {
-            I.m2m_ptr[l] = int(m2m_cells.size());
-            if (l >= 2)
-                for (int c = T.level_start[l]; c < T.level_start[l + 1]; ++c)
-                    if (!T.is_leaf(c) && sub_pieces[c] > 0) m2m_cells.push_back(c);
-        }
-        I.m2m_ptr[T.depth + 1] = int(m2m_cells.size());
+        up_need.assign(nC, 0);
+        for (int l = 2; l <= T.depth; ++l)
+            for (int c = T.level_start[l]; c < T.level_start[l + 1]; ++c)
+                if (!T.is_leaf(c) && sub_pieces[c] > 0) {
+                    m2m_cells.push_back(c);
+                    for (int q = 0; q < 4; ++q) {
+                        const int d = T.child0[c] + q;
+                        if (!T.is_leaf(d) && sub_pieces[d] > 0) up_need[c]++;
+                    }
+                }
+        // deepest first: their chains to the top are the longest
+        for (size_t i = m2m_cells.size(); i-- > 0;)
+            if (up_need[m2m_cells[i]] == 0) up_starts.push_back(m2m_cells[i]);
         std::vector<int> stack, lv;
         for (int a : m2m_cells) {
             lv.clear();
@@ -973,25 +1014,30 @@ dc_status Fmm::build(const dc_options &opt, const Geometry &G, const DevGeom &D,
     for (int k = 0; k < 32; ++k)
         for (int j = 0; j <= k; ++j) binom32[k * 32 + j] = (float)binom(k, j);
     auto make_sched = [&](Schedule &sc, bool nodes_only, std::vector<int> &m2l_c,
-                          std::vector<int> &p2l_c, std::vector<int> &l2l_c, std::vector<int> &walk_c) {
-        sc.l2l_ptr.assign(T.depth + 2, 0);
-        for (int l = 0; l <= T.depth; ++l) {
-            sc.l2l_ptr[l] = int(l2l_c.size());
-            if (l < 2) continue;
+                          std::vector<int> &p2l_c, std::vector<int2> &l2l_c, std::vector<int> &walk_c) {
+        sc.l2l_ptr.clear();
+        for (int l = 2; l <= T.depth; ++l) {
+            if (l % 2 == 0) sc.l2l_ptr.push_back(int(l2l_c.size()));
             for (int c = T.level_start[l]; c < T.level_start[l + 1]; ++c) {
                 if (nodes_only && sub_nodes[c] == 0) continue;
-                l2l_c.push_back(c);
+                if (l % 2 == 0) {
+                    int mask = 0;
+                    for (int q = 0; q < 4 && !T.is_leaf(c); ++q)
+                        if (!nodes_only || sub_nodes[T.child0[c] + q] > 0) mask |= 1 << q;
+                    l2l_c.push_back(make_int2(c, mask));
+                }
                 if (T.v_ptr[c + 1] > T.v_ptr[c]) m2l_c.push_back(c);
                 if (T.x_ptr[c + 1] > T.x_ptr[c]) p2l_c.push_back(c);
                 if (T.is_leaf(c)) walk_c.push_back(c);
             }
         }
-        sc.l2l_ptr[T.depth + 1] = int(l2l_c.size());
+        sc.l2l_ptr.push_back(int(l2l_c.size()));
         sc.n_m2l = int(m2l_c.size());
         sc.n_p2l = int(p2l_c.size());
         sc.n_walk = int(walk_c.size());
     };
-    std::vector<int> am2l, ap2l, al2l, aw, nm2l, np2l, nl2l, nw;
+    std::vector<int> am2l, ap2l, aw, nm2l, np2l, nw;
+    std::vector<int2> al2l, nl2l;
     phase(0);   // quadtree, lists, tables, multi-level M2M chunks
     // the FP32 form's host arrays (tree and discretisation only) on a helper
     // thread while the schedules, preconditioner and coefficients are built
@@ -1213,7 +1259,9 @@ dc_status Fmm::build(const dc_options &opt, const Geometry &G, const DevGeom &D,
     UP(I.logw64, logw64);
     UP(I.plen64, plen64);
     UP(I.v_code, vcode);
-    UP(I.m2m_cells, m2m_cells);
+    UP(I.up_starts, up_starts);
+    UP(I.up_need, up_need);
+    I.n_up = int(up_starts.size());
     {   // list-1 pieces of every leaf, flattened in list order: the offsets
         // here, the piece and segment numbers by uf_fill_kernel
         std::vector<int> ufp(nC + 1, 0);
@@ -1292,8 +1340,18 @@ dc_status Fmm::build(const dc_options &opt, const Geometry &G, const DevGeom &D,
         (e = I.L.alloc((size_t)nC * 3 * I.P1)) != cudaSuccess ||
         (e = upload_cd(I.base64, base, st)) != cudaSuccess ||
         (e = upload(I.baseff, to_ff(base), st)) != cudaSuccess ||
-        (e = upload(I.m2mff, to_ff(m2m), st)) != cudaSuccess ||
-        (e = upload(I.l2lff, to_ff(l2l), st)) != cudaSuccess ||
+        (e = upload(I.m2mff, to_ff(lane_order(m2m, true, I.P1)), st)) != cudaSuccess ||
+        (e = upload(I.l2lff, to_ff(lane_order(l2l, false, I.P1)), st)) != cudaSuccess ||
+        (e = I.Mff.alloc((size_t)nC * 3 * I.P1)) != cudaSuccess ||
+        (e = I.Lff.alloc((size_t)nC * 3 * I.P1)) != cudaSuccess ||
+        (e = I.Lxff.alloc((size_t)nC * 3 * I.P1)) != cudaSuccess ||
+        (e = cudaMemsetAsync(I.Mff.ptr, 0, I.Mff.bytes(), st)) != cudaSuccess ||   // cells without pieces stay zero
+        (e = cudaMemsetAsync(I.M.ptr, 0, I.M.bytes(), st)) != cudaSuccess ||
+        (e = I.up_arrived.alloc((size_t)nC)) != cudaSuccess ||
+        (e = cudaMemsetAsync(I.up_arrived.ptr, 0, I.up_arrived.bytes(), st)) != cudaSuccess ||
+        (!I.p2l_stream && (e = cudaStreamCreateWithFlags(&I.p2l_stream, cudaStreamNonBlocking)) != cudaSuccess) ||
+        (!I.p2l_ev[0] && (e = cudaEventCreateWithFlags(&I.p2l_ev[0], cudaEventDisableTiming)) != cudaSuccess) ||
+        (!I.p2l_ev[1] && (e = cudaEventCreateWithFlags(&I.p2l_ev[1], cudaEventDisableTiming)) != cudaSuccess) ||
         (e = upload(I.m2m32i, to_f2(m2mi), st)) != cudaSuccess ||
         (e = upload(I.l2l32i, to_f2(l2li), st)) != cudaSuccess ||
         (e = upload(I.base32i, to_f2(basei), st)) != cudaSuccess ||
@@ -1354,8 +1412,6 @@ dc_status Fmm::build(const dc_options &opt, const Geometry &G, const DevGeom &D,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)passes::p2m_smem<double>(I.P1));
     cudaFuncSetAttribute(passes::p2l_flat_kernel<double, passes::PiecesF64>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)passes::p2l_flat_smem<double>(I.P1));
-    cudaFuncSetAttribute(passes::m2m_ff_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)passes::mlff_smem(I.P1));
     phase(2);   // two-level preconditioner
     // The node near / far coefficients on a helper thread and the tree's
     // stream (free again) while the stored rows and the FP32 form are built
@@ -1693,7 +1749,7 @@ static dc_status launch_render(Fmm::Impl &I, int n_tiles, void *rgb, int rgb_dty
         }
         eval_tiles_kernel<<<std::min(n_tiles, I.n_sms * kFfBlocksPerSM), kFfThreads, 0, st>>>(
             I.dt(), I.tiles.ptr, n_tiles, I.render_queue.ptr, I.vps.ptr, I.P1, I.plen64.ptr, I.uf_ptr.ptr, I.uf_idx.ptr,
-            I.M.ptr, I.L.ptr, sbar, mbar, rgb, rgb_dtype, rgb8);
+            I.Mff.ptr, I.Lff.ptr, sbar, mbar, rgb, rgb_dtype, rgb8);
         note_launch();
         e = cudaGetLastError();
     }

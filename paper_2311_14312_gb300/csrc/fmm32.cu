@@ -102,7 +102,7 @@ __global__ void interp32_kernel(const float2 *__restrict__ lam, const double *__
 #define DC_BIG_COEF 50.0
 #endif
 constexpr double kBigCoef = DC_BIG_COEF;
-__global__ void big_coef_kernel(const double2 *__restrict__ L, const double2 *__restrict__ M, int n,
+__global__ void big_coef_kernel(const float4 *__restrict__ L, const float4 *__restrict__ M, int n,
                                 int P1, unsigned char *__restrict__ hL, unsigned char *__restrict__ hM) {
     // one warp per cell, lanes over the coefficients (coalesced); magnitudes in FP32, since this
     // is a threshold test and FP64 hypot runs at 1/64 of the FP32 rate
@@ -110,12 +110,12 @@ __global__ void big_coef_kernel(const double2 *__restrict__ L, const double2 *__
     if (c >= n) return;
     float bl = 0.f, bm = 0.f;
     for (int ch = 0; ch < 3; ++ch) {
-        const double2 *l = L + ((size_t)c * 3 + ch) * P1, *m = M + ((size_t)c * 3 + ch) * P1;
+        const float4 *l = L + ((size_t)c * 3 + ch) * P1, *m = M + ((size_t)c * 3 + ch) * P1;
         float sl = 0.f, sm = 0.f;
         for (int k = lane; k < P1; k += 32) {
-            const double2 lk = l[k], mk = m[k];
-            sl += hypotf((float)lk.x, (float)lk.y);
-            sm += (k == 0 ? 10.f : 1.f) * hypotf((float)mk.x, (float)mk.y);
+            const float4 lk = l[k], mk = m[k];
+            sl += hypotf(lk.x, lk.y);
+            sm += (k == 0 ? 10.f : 1.f) * hypotf(mk.x, mk.y);
         }
         for (int o = 16; o > 0; o >>= 1) {
             sl += __shfl_xor_sync(0xffffffffu, sl, o);
@@ -143,7 +143,7 @@ __global__ void near_centre_kernel(const int *__restrict__ uf_ptr, const int *__
                                    const int *__restrict__ pseg, const float *__restrict__ pw,
                                    const float *__restrict__ plen, const unsigned char *__restrict__ heavy,
                                    const float *__restrict__ sb, const float *__restrict__ iw, int nC, int P1,
-                                   double2 *__restrict__ L) {
+                                   float4 *__restrict__ L) {
     const int cell = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (cell >= nC || uf_ptr[cell + 1] == uf_ptr[cell]) return;
     const float iwf = iw[cell];
@@ -161,21 +161,26 @@ __global__ void near_centre_kernel(const int *__restrict__ uf_ptr, const int *__
     if (lane == 0) {
         const double iwd = (double)iwf;
         const double k = -6.283185307179586477 * log(iwd) / iwd;   // 2 pi rho log(rho)
-        for (int ch = 0; ch < 3; ++ch) L[((size_t)cell * 3 + ch) * P1].x += k * acc[ch];
+        for (int ch = 0; ch < 3; ++ch) {
+            float4 &l = L[((size_t)cell * 3 + ch) * P1];
+            const double v = ((double)l.x + (double)l.z) + k * acc[ch];
+            l.x = (float)v;
+            l.z = (float)(v - (double)l.x);
+        }
     }
 }
 
 // FP32 copies of the expansions for the evaluation: M with M_k / k in the
 // place of M_k (k >= 1), the factor of Eq. 61, and L.
-__global__ void narrow_kernel(const double2 *__restrict__ M, const double2 *__restrict__ L, float2 *__restrict__ M32,
+__global__ void narrow_kernel(const float4 *__restrict__ M, const float4 *__restrict__ L, float2 *__restrict__ M32,
                               float2 *__restrict__ L32, int P1, size_t n) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int k = (int)(i % P1);
     const float ik = k > 0 ? 1.f / k : 1.f;
-    const double2 m = M[i], l = L[i];
-    M32[i] = make_float2((float)m.x * ik, (float)m.y * ik);
-    L32[i] = make_float2((float)l.x, (float)l.y);
+    const float4 m = M[i], l = L[i];   // normalised: the hi parts are the values rounded
+    M32[i] = make_float2(m.x * ik, m.y * ik);
+    L32[i] = make_float2(l.x, l.y);
 }
 
 // heavy[i] = 1 when max_c |sigma_bar| w len or |mu_bar| w len of piece i
@@ -219,7 +224,7 @@ struct EvalArgs32 {
     // FP64 path for heavy pieces and big-coefficient cells (pixel mode)
     const double *sb64, *mb64;
     const unsigned char *heavy, *hL, *hM;
-    const double2 *M64, *L64;
+    const float4 *M64, *L64;   // float-float: re hi, im hi, re lo, im lo
 
     // persistent launch: the item counter (zero at launch) and the item count
     int *queue;
@@ -230,6 +235,11 @@ struct EvalArgs32 {
     const int *own1, *own2, *perm;
     double *out;
 };
+
+// the FP64 value of a float-float coefficient
+__device__ __forceinline__ double2 ff_value(float4 v) {
+    return make_double2((double)v.x + (double)v.z, (double)v.y + (double)v.w);
+}
 
 __device__ __forceinline__ unsigned char quant8(float v) {
     v = fminf(fmaxf(v, 0.f), 1.f);
@@ -294,12 +304,13 @@ __device__ __forceinline__ void eval32_item(const EvalArgs32 &a, int item) {
         if (a.hL && a.hL[leaf]) {
             const double iw = 1.0 / a.t64.cw[leaf];
             const double zx = (qx64 - cxB) * iw, zy = (qy64 - cyB) * iw;
-            const double2 *Lc = a.L64 + (size_t)leaf * 3 * P1;
+            const float4 *Lc = a.L64 + (size_t)leaf * 3 * P1;
             for (int ch = 0; ch < 3; ++ch) {
-                double sx = Lc[ch * P1 + P1 - 1].x, sy = Lc[ch * P1 + P1 - 1].y;
-                for (int k = P1 - 2; k >= 0; --k) {
-                    double nx = sx * zx - sy * zy + Lc[ch * P1 + k].x;
-                    sy = sx * zy + sy * zx + Lc[ch * P1 + k].y;
+                double sx = 0.0, sy = 0.0;
+                for (int k = P1 - 1; k >= 0; --k) {
+                    const double2 l = ff_value(Lc[ch * P1 + k]);
+                    double nx = sx * zx - sy * zy + l.x;
+                    sy = sx * zy + sy * zx + l.y;
                     sx = nx;
                 }
                 (ch == 0 ? h0 : ch == 1 ? h1 : h2) += sx * kInv2Pi;
@@ -327,17 +338,18 @@ __device__ __forceinline__ void eval32_item(const EvalArgs32 &a, int item) {
                 const double d = 1.0 / (zx * zx + zy * zy);
                 const double izx = zx * d, izy = -zy * d;
                 const double lz = 0.5 * log(zx * zx + zy * zy) + log(a.t64.cw[src]);
-                const double2 *Ms = a.M64 + (size_t)src * 3 * P1;
+                const float4 *Ms = a.M64 + (size_t)src * 3 * P1;
                 for (int ch = 0; ch < 3; ++ch) {
-                    const double2 *m = Ms + ch * P1;
-                    double sx = m[P1 - 1].x / (P1 - 1), sy = m[P1 - 1].y / (P1 - 1);
-                    for (int k = P1 - 2; k >= 1; --k) {
-                        double nx = sx * izx - sy * izy + m[k].x / k;
-                        sy = sx * izy + sy * izx + m[k].y / k;
+                    const float4 *m = Ms + ch * P1;
+                    double sx = 0.0, sy = 0.0;
+                    for (int k = P1 - 1; k >= 1; --k) {
+                        const double2 v = ff_value(m[k]);
+                        double nx = sx * izx - sy * izy + v.x / k;
+                        sy = sx * izy + sy * izx + v.y / k;
                         sx = nx;
                     }
                     double rx = sx * izx - sy * izy;
-                    (ch == 0 ? h0 : ch == 1 ? h1 : h2) += (rx - lz * m[0].x) * kInv2Pi;
+                    (ch == 0 ? h0 : ch == 1 ? h1 : h2) += (rx - lz * ff_value(m[0]).x) * kInv2Pi;
                 }
                 continue;
             }
@@ -833,12 +845,12 @@ cudaError_t Fmm::Impl::prepare_render32(const double *sb, const double *mb, cuda
     }
     near_centre_kernel<<<(unsigned)(((size_t)nC * 32 + th - 1) / th), th, 0, st>>>(
         uf_ptr.ptr, uf_idx.ptr, pseg.ptr, pw32.ptr, plen32.ptr, np > 0 ? heavy.ptr : nullptr, sbar32.ptr, iw32.ptr, nC,
-        P1, L.ptr);
+        P1, Lff.ptr);
     note_launch();
-    big_coef_kernel<<<(unsigned)(((size_t)nC * 32 + th - 1) / th), th, 0, st>>>(L.ptr, M.ptr, nC, P1, heavyL.ptr, heavyM.ptr);
+    big_coef_kernel<<<(unsigned)(((size_t)nC * 32 + th - 1) / th), th, 0, st>>>(Lff.ptr, Mff.ptr, nC, P1, heavyL.ptr, heavyM.ptr);
     note_launch();
     const size_t n = (size_t)nC * 3 * P1;
-    narrow_kernel<<<(unsigned)((n + th - 1) / th), th, 0, st>>>(M.ptr, L.ptr, M32.ptr, L32.ptr, P1, n);
+    narrow_kernel<<<(unsigned)((n + th - 1) / th), th, 0, st>>>(Mff.ptr, Lff.ptr, M32.ptr, L32.ptr, P1, n);
     note_launch();
     return cudaGetLastError();
 }
@@ -1063,8 +1075,8 @@ cudaError_t Fmm::Impl::render_tiles32(int n_tiles, void *rgb, int rgb_dtype,
     a.use_m = 1;
     a.hL = heavyL.ptr;
     a.hM = heavyM.ptr;
-    a.M64 = M.ptr;
-    a.L64 = L.ptr;
+    a.M64 = Mff.ptr;
+    a.L64 = Lff.ptr;
     a.vps = vps.ptr;
     a.rgb = rgb;
     a.rgb_dtype = rgb_dtype;
@@ -1091,8 +1103,8 @@ cudaError_t Fmm::Impl::eval_points32_at(const Tile *items, int n_items, const do
 
     a.hL = heavyL.ptr;
     a.hM = heavyM.ptr;
-    a.M64 = M.ptr;
-    a.L64 = L.ptr;
+    a.M64 = Mff.ptr;
+    a.L64 = Lff.ptr;
     a.t = dt32();
     a.t64 = dt();
     a.items = items;

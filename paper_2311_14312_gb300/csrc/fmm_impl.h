@@ -93,8 +93,9 @@ inline int tile_side(double pixels, int cap) {
 // Cells that need incoming expansions for one set of targets (all cells for
 // pixels; the cells above the nodes for the matvec), by pass.
 struct Schedule {
-    DevBuf<int> m2l, p2l, l2l;        // cells with list 2 / list 4; cells per level
-    std::vector<int> l2l_ptr;         // [depth + 2] offsets into l2l by level
+    DevBuf<int> m2l, p2l;             // cells with list 2 / list 4
+    DevBuf<int2> l2l;                 // cells of the even levels, with the mask of their scheduled children
+    std::vector<int> l2l_ptr;         // offsets into l2l by even level (2, 4, ...)
     DevBuf<int> walk;                 // leaves whose incoming expansion is needed
     DevBuf<int> chains;               // per walk leaf: length, then itself and its ancestors to level 2
     int n_m2l = 0, n_p2l = 0, n_walk = 0;
@@ -140,7 +141,7 @@ struct Fmm::Impl {
     bool near_ready = false;
     DevBuf<double> near_g64, near_f64;   // while they are built (near and far both stored: float-float)
     DevBuf<float2> near_gff, near_fff, dens_ff;
-    DevBuf<float4> farff, Lff, Mff;
+    DevBuf<float4> farff;
     DevBuf<float> near_g32;
     cudaError_t build_near(cudaStream_t st);
     // far-field coefficients of the node targets: (1 + list-3 length) blocks
@@ -163,7 +164,8 @@ struct Fmm::Impl {
     DevBuf<float2> p2m_g32;
     cudaError_t build_rows(cudaStream_t st);
     // FP64 tables and expansions
-    DevBuf<double2> m2m, l2l, m2l, M, L;
+    DevBuf<double2> m2m, l2l, m2l, M, L;   // M, L: FP64 values of Mff, Lff where a kernel reads those (widen)
+    DevBuf<float4> Mff, Lff, Lxff;    // the FP64 passes' expansions in float-float; Lxff: list-2 and list-4 terms
     DevBuf<double> sbar, mbar;
     DevBuf<RTile> tiles;              // the render's tiles, by decreasing estimated cost
     DevBuf<int> render_queue;         // the persistent render's tile counter
@@ -185,9 +187,8 @@ struct Fmm::Impl {
     DevBuf<int> pinfo;
     // pass schedules and tables of the templated passes
     Schedule sched_all, sched_nodes;
-    DevBuf<int> m2m_cells, v_code;
+    DevBuf<int> v_code;
     DevBuf<int> uf_ptr, uf_idx, uf_seg;   // list-1 pieces per leaf, flattened, and their segments
-    std::vector<int> m2m_ptr;         // [depth + 2]: inner cells with pieces, by level
     // one-launch upward pass of the FP32 operator: chunks (ancestor, first
     // pair, pairs, slot), reductions (cell, first slot, slots), leaves of the
     // pairs, C(k, j)
@@ -201,7 +202,14 @@ struct Fmm::Impl {
     int walk_nmax = 1;                // longest walk chain (levels 2 .. depth)
     DevBuf<double2> base64, Lm2l;
     DevBuf<float4> baseff;            // base M2L tables in float-float
-    DevBuf<float4> m2mff, l2lff;      // M2M / L2L tables in float-float
+    DevBuf<float4> m2mff, l2lff;      // M2M / L2L tables in float-float, in lane order (passes.cuh)
+    // one-launch upward pass: its first cells, inner children with pieces per
+    // cell, and how many of those have been computed (zero between passes)
+    DevBuf<int> up_starts, up_need, up_arrived;
+    int n_up = 0;
+    // list 4 beside the upward pass
+    cudaStream_t p2l_stream = nullptr;
+    cudaEvent_t p2l_ev[2] = {nullptr, nullptr};
     DevBuf<float2> base32, Lm2l32;
     // the FP32 operator inside GMRES runs at a lower order p_inner (its
     // accuracy only has to beat the inner tolerance; the FP64 residual at
@@ -268,6 +276,9 @@ struct Fmm::Impl {
         if (pre_stream) cudaStreamDestroy(pre_stream);
         if (tree_stream) cudaStreamDestroy(tree_stream);
         if (pre_ev) cudaEventDestroy(pre_ev);
+        if (p2l_stream) cudaStreamDestroy(p2l_stream);
+        for (auto &ev : p2l_ev)
+            if (ev) cudaEventDestroy(ev);
         for (auto &ev : fork_ev)
             if (ev) cudaEventDestroy(ev);
     }
@@ -278,6 +289,7 @@ struct Fmm::Impl {
     cudaError_t passes(const double *sb, const double *mb, int use_s, int use_m, cudaStream_t st,
                        const Schedule &sc);
     cudaError_t apply_nodes(const double *x, double *y, bool single, cudaStream_t st);
+    cudaError_t widen(cudaStream_t st);   // M, L from Mff, Lff
     // FP32 (fmm32.cu)
     // host arrays of the FP32 form that depend on the (pruned) tree and the
     // discretisation alone: built on a helper thread during the schedules

@@ -7,7 +7,7 @@
 //               shared memory, then one thread per coefficient summing the
 //               chunk in order (deterministic)
 //               (or from stored per-piece coefficient rows)
-//  m2m_kernel   per level, parent from its 4 children (Eq. 71)
+//  m2m_up_kernel  parent from its 4 children (Eq. 71), float-float, one launch
 //  m2m_multi_kernel  every inner cell straight from its leaves (all levels
 //               in one launch, no chain of dependent levels)
 //  m2l_kernel   all cells at once, persistent blocks: list 2 (Eq. 69) with
@@ -17,7 +17,7 @@
 //               conjugate analogue, u in {1, i, -1, -i}
 //  p2l_kernel   cells with a list 4: incoming coefficients of segments
 //               (Eq. 62/78/79), chunked like p2m
-//  l2l_kernel   per level: L = L_m2l + L2L(parent) (Eq. 73)
+//  l2l_two_kernel  two levels a launch: L = L_m2l + L2L(parent) (Eq. 73), float-float
 //  walk_kernel  the same recursion for listed leaves only, walking down from
 //               each leaf's level-2 ancestor (one launch for all levels)
 #pragma once
@@ -228,34 +228,6 @@ __global__ void __launch_bounds__(kChunk) p2m_kernel(TreeView<T> t, PS ps, const
 }
 
 // ---------------------------------------------------------------- M2M --
-// One level: each listed cell's expansion from its four children (Eq. 71),
-// one warp per cell, lane k holds coefficient k (P1 <= 32).
-constexpr int kLevelWarps = 4;
-
-template <typename T>
-__global__ void __launch_bounds__(32 * kLevelWarps) m2m_kernel(const int *__restrict__ child0,
-                                                               const int *__restrict__ cells, int n, int P1,
-                                                               const typename V2<T>::type *__restrict__ tab,
-                                                               typename V2<T>::type *__restrict__ M) {
-    using C = typename V2<T>::type;
-    const int idx = blockIdx.x * kLevelWarps + (threadIdx.x >> 5);
-    const int k = threadIdx.x & 31;
-    if (idx >= n || k >= P1) return;
-    const int cell = cells[idx];
-    const int ch0 = child0[cell];
-    C acc[3];
-    for (int c = 0; c < 3; ++c) acc[c] = mk<T>(0, 0);
-    for (int q = 0; q < 4; ++q) {
-        const C *Tq = tab + ((size_t)q * P1 + k) * P1;
-        const C *src = M + (size_t)(ch0 + q) * 3 * P1;
-        for (int j = 0; j <= k; ++j) {
-            C tq = Tq[j];
-            for (int c = 0; c < 3; ++c) cfma(acc[c], tq, src[c * P1 + j]);
-        }
-    }
-    for (int c = 0; c < 3; ++c) M[((size_t)cell * 3 + c) * P1 + k] = acc[c];
-}
-
 // M2M from each leaf straight to every listed ancestor, all levels in one
 // launch: Eq. 71 with the shift d = (c_leaf - c_anc) / w_anc and the scale
 // rho = w_leaf / w_anc of the width-scaled basis (pair_geo = (d, rho, 0)),
@@ -630,133 +602,158 @@ __device__ __forceinline__ float4 ff_rot(float4 v, int n) {
 }
 __device__ __forceinline__ float4 ff_conj(float4 v) { return make_float4(v.x, -v.y, v.z, -v.w); }
 
-// Per-level M2M (Eq. 71) and L2L (Eq. 73) of the FP64 passes in float-float
-// (the tables of m2m_kernel / l2l_kernel stored as float-float): one warp per
-// cell, lane k holds coefficient k; the FP64 inputs (children's moments, the
-// parent's local expansion) are converted once per cell into shared memory,
-// so the inner loops run on the FP32 pipes only.
-// M2M lanes: coefficient k and P1 - 1 - k share a lane (k + 1 and P1 - k
-// terms, P1 + 1 together), and the two half-warps take children 0, 1 and
-// 2, 3, so 2 ceil(P1 / 2) lanes carry equal loads; the halves' sums are
-// added at the end.  The four quadrant tables are staged in shared memory.
+// M2M (Eq. 71) and L2L (Eq. 73) of the FP64 passes in float-float.  The
+// expansions are kept as float-float complex values (float4: re hi, im hi, re
+// lo, im lo), so no kernel of the passes touches the FP64 pipe for them.
+//
+// What bounded these passes was latency: a launch per level, and in it a
+// warp per cell walking 6,000 instructions.  Here 12 warps share a cell: a
+// warp takes a channel and a child (quadrant), 16 lanes the outputs in pairs
+// (coefficient kk and P1 - 1 - kk have P1 + 1 terms together, so the lanes
+// carry equal loads), the two halves of the warp the even and the odd terms.
+// The tables are stored in the order the lanes read them ([quadrant][step]
+// [lane], zero where a lane has no term).  On the 200-curve drawing (11,529
+// cells, 13 levels, order 24) the upward pass took 229 us in 11 launches and
+// the downward one 204 us in 12; see Fmm::Impl::passes for the times now.
 __device__ __forceinline__ float4 ff_shfl_xor(float4 v, int m) {
     return make_float4(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m),
                        __shfl_xor_sync(0xffffffffu, v.z, m), __shfl_xor_sync(0xffffffffu, v.w, m));
 }
-
-__device__ __forceinline__ double2 ff_to_double(float4 a) {
-    return make_double2((double)a.x + (double)a.z, (double)a.y + (double)a.w);
+// the same value with the lo parts below half a unit of the hi parts
+__device__ __forceinline__ float4 ff_norm(float4 a) {
+    const float x = __fadd_rn(a.x, a.z), y = __fadd_rn(a.y, a.w);
+    return make_float4(x, y, __fsub_rn(a.z, __fsub_rn(x, a.x)), __fsub_rn(a.w, __fsub_rn(y, a.y)));
 }
 
-// shared memory of m2m_ff_kernel: the four quadrant tables and each warp's
-// staged children
-inline size_t mlff_smem(int P1) { return (4 * (size_t)P1 * P1 + 4 * 4 * 3 * (size_t)P1) * sizeof(float4); }
-
-static __global__ void __launch_bounds__(128) m2m_ff_kernel(const int *__restrict__ child0,
-                                                            const int *__restrict__ cells, int n, int P1,
-                                                            const float4 *__restrict__ tab,
-                                                            double2 *__restrict__ M) {
-    extern __shared__ unsigned char smem_raw[];
-    float4 *tabs = reinterpret_cast<float4 *>(smem_raw);   // [4][P1][P1]
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nM = 3 * P1;
-    float4 *smw = tabs + 4 * P1 * P1 + w * 4 * nM;          // this warp's 4 children
-    stage_async(tabs, tab, 4 * P1 * P1, threadIdx.x, blockDim.x);
-    cp_async_commit();
-    const int idx = blockIdx.x * 4 + w;
-    const bool live = idx < n;
-    const int cell = live ? cells[idx] : 0;
-    if (live) {
-        const double2 *src = M + (size_t)child0[cell] * nM;   // the 4 children are contiguous
-        // four loads in flight per lane, then the conversions
-        for (int i0 = lane; i0 < 4 * nM; i0 += 4 * 32) {
-            double2 v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int i = i0 + 32 * u;
-                v[u] = i < 4 * nM ? src[i] : make_double2(0.0, 0.0);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int i = i0 + 32 * u;
-                if (i < 4 * nM) smw[i] = ff_from(v[u]);
-            }
-        }
-    }
-    cp_async_wait<0>();
-    __syncthreads();
-    if (!live) return;
-    tab = tabs;
-    const int kk = lane & 15, h = lane >> 4;
-    const int k1 = kk, k2 = P1 - 1 - kk;
-    const bool on = k1 <= k2, two = k1 < k2;
+constexpr int kPairThreads = 384, kPairLanes = 16;
+// Step i of lane kk, 0 <= i <= P1, 2 kk < P1: the output and the input index.
+//   up (M2M):   k = kk,           j = i           for i <= kk,
+//               k = P1 - 1 - kk,  j = i - kk - 1  beyond
+//   down (L2L): l = kk,           k = kk + i      for i < P1 - kk,
+//               l = P1 - 1 - kk,  k = i - 1       beyond
+__host__ __device__ __forceinline__ int pair_switch(bool up, int P1, int kk) { return up ? kk + 1 : P1 - kk; }
+__host__ __device__ __forceinline__ int pair_in(bool up, int P1, int kk, int i) {
+    const int n1 = pair_switch(up, P1, kk);
+    return up ? (i < n1 ? i : i - n1) : (i < n1 ? kk + i : i - 1);
+}
+// the two outputs of lane kk from the values v (shared memory), every
+// second step from h on; tab: the quadrant's table
+template <bool UP>
+__device__ __forceinline__ void pair_sums(const float4 *__restrict__ tab, const float4 *v, int P1, int kk, int h,
+                                          float4 &a1, float4 &a2) {
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 a1[3] = {z, z, z}, a2[3] = {z, z, z};
-    if (on)
-        for (int q = 2 * h; q < 2 * h + 2; ++q) {
-            const float4 *mq = smw + q * nM;
-            const float4 *T1 = tab + ((size_t)q * P1 + k1) * P1;
-            for (int j = 0; j <= k1; ++j) {
-                const float4 tq = T1[j];
-                for (int c = 0; c < 3; ++c) ff_cfma(a1[c], tq, mq[c * P1 + j]);
-            }
-            if (two) {
-                const float4 *T2 = tab + ((size_t)q * P1 + k2) * P1;
-                for (int j = 0; j <= k2; ++j) {
-                    const float4 tq = T2[j];
-                    for (int c = 0; c < 3; ++c) ff_cfma(a2[c], tq, mq[c * P1 + j]);
-                }
-            }
+    a1 = a2 = z;
+    if (2 * kk >= P1) return;
+    const int n1 = pair_switch(UP, P1, kk);
+    float4 acc = z;
+    bool second = false;
+    for (int i = h; i <= P1; i += 2) {
+        if (!second && i >= n1) {
+            a1 = acc;
+            acc = z;
+            second = true;
         }
-    for (int c = 0; c < 3; ++c) {
-        ff_cadd(a1[c], ff_shfl_xor(a1[c], 16));
-        ff_cadd(a2[c], ff_shfl_xor(a2[c], 16));
+        ff_cfma(acc, __ldg(tab + i * kPairLanes + kk), v[pair_in(UP, P1, kk, i)]);
     }
-    if (h != 0 || !on) return;
-    for (int c = 0; c < 3; ++c) {
-        M[((size_t)cell * 3 + c) * P1 + k1] = ff_to_double(a1[c]);
-        if (two) M[((size_t)cell * 3 + c) * P1 + k2] = ff_to_double(a2[c]);
+    if (second) a2 = acc;
+    else a1 = acc;
+}
+
+// Upward pass in one launch: block b computes the inner cell starts[b] (one
+// without inner children that hold pieces) from its four children, and the
+// block that brings the last of a parent's inner children goes on with the
+// parent (arrived counts them against need, and is left at zero).  Nothing
+// waits; a cell's sum runs over its children in a fixed order whichever block
+// computes it.
+static __global__ void __launch_bounds__(kPairThreads) m2m_up_kernel(const int *__restrict__ child0,
+                                                                     const int *__restrict__ parent,
+                                                                     const int *__restrict__ starts,
+                                                                     const int *__restrict__ need,
+                                                                     int *__restrict__ arrived, int P1,
+                                                                     const float4 *__restrict__ tab, float4 *M) {
+    __shared__ float4 v[4 * 3 * 32];
+    __shared__ float4 part[12][2][kPairLanes];
+    __shared__ int next;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int c = warp >> 2, q = warp & 3, kk = lane & 15, h = lane >> 4;
+    const int nM = 3 * P1;
+    int cell = starts[blockIdx.x];
+    while (true) {
+        const float4 *src = M + (size_t)child0[cell] * nM;   // the 4 children are contiguous
+        for (int i = tid; i < 4 * nM; i += kPairThreads) v[i] = __ldcg(src + i);
+        __syncthreads();
+        float4 a1, a2;
+        pair_sums<true>(tab + (size_t)q * (P1 + 1) * kPairLanes, v + (q * 3 + c) * P1, P1, kk, h, a1, a2);
+        __syncwarp();
+        ff_cadd(a1, ff_shfl_xor(a1, 16));
+        ff_cadd(a2, ff_shfl_xor(a2, 16));
+        if (h == 0) {
+            part[warp][0][kk] = a1;
+            part[warp][1][kk] = a2;
+        }
+        __syncthreads();
+        if (tid < nM) {
+            const int ch = tid / P1, k = tid - ch * P1, k2 = P1 - 1 - k;
+            const int o = k <= k2 ? 0 : 1, l = k <= k2 ? k : k2;
+            float4 a = part[4 * ch][o][l];
+            for (int i = 1; i < 4; ++i) ff_cadd(a, part[4 * ch + i][o][l]);
+            M[(size_t)cell * nM + tid] = ff_norm(a);
+        }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            const int p = parent[cell], n = need[p];
+            next = -1;
+            if (n > 0 && atomicAdd(arrived + p, 1) == n - 1) {
+                arrived[p] = 0;
+                next = p;
+            }
+            __threadfence();
+        }
+        __syncthreads();
+        cell = next;
+        if (cell < 0) break;
     }
 }
 
-static __global__ void __launch_bounds__(128) l2l_ff_kernel(TreeView<double> t, const int *__restrict__ cells, int n,
-                                                            int level, int P1, const float4 *__restrict__ tab,
-                                                            const double2 *__restrict__ Lm2l,
-                                                            double2 *__restrict__ L) {
-    __shared__ float4 sp[4][3 * 32];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    const int idx = blockIdx.x * 4 + w;
-    if (idx >= n) return;
-    const int cell = cells[idx];
+// Downward pass, two levels a launch: block b computes cell cells[b].x from
+// its parent (up = 0: level 2, which has none) and then those of its four
+// children whose bit is set in cells[b].y; Lx holds the list-2 and list-4
+// terms.
+static __global__ void __launch_bounds__(kPairThreads) l2l_two_kernel(const int *__restrict__ child0,
+                                                                      const int *__restrict__ parent,
+                                                                      const int *__restrict__ quad,
+                                                                      const int2 *__restrict__ cells, int up, int P1,
+                                                                      const float4 *__restrict__ tab,
+                                                                      const float4 *__restrict__ Lx, float4 *L) {
+    __shared__ float4 sp[3 * 32], sc[3 * 32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, kk = lane & 15, h = lane >> 4;
     const int nM = 3 * P1;
-    const bool up = level >= 3;
-    if (up) {
-        const double2 *src = L + (size_t)t.parent[cell] * nM;
-        for (int i = l; i < nM; i += 32) sp[w][i] = ff_from(src[i]);
-    }
-    __syncwarp();
-    if (l >= P1) return;
-    float4 acc[3];
-    for (int c = 0; c < 3; ++c) acc[c] = ff_from(Lm2l[((size_t)cell * 3 + c) * P1 + l]);
-    if (up) {
-        const float4 *Tq = tab + ((size_t)t.quad[cell] * P1 + l) * P1;
-        int k = l;
-        for (; k + 4 <= P1; k += 4) {   // four table loads in flight
-            float4 tq[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) tq[u] = Tq[k + u];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                for (int c = 0; c < 3; ++c) ff_cfma(acc[c], tq[u], sp[w][c * P1 + k + u]);
+    const int cell = cells[blockIdx.x].x, mask = cells[blockIdx.x].y;
+    auto step = [&](int to, int q, int c, const float4 *v, bool from_parent, float4 *keep) {
+        float4 a1 = make_float4(0.f, 0.f, 0.f, 0.f), a2 = a1;
+        if (from_parent) pair_sums<false>(tab + (size_t)q * (P1 + 1) * kPairLanes, v + c * P1, P1, kk, h, a1, a2);
+        __syncwarp();
+        ff_cadd(a1, ff_shfl_xor(a1, 16));
+        ff_cadd(a2, ff_shfl_xor(a2, 16));
+        // half 0 finishes the first output, half 1 the second
+        const int l = h == 0 ? kk : P1 - 1 - kk;
+        if (2 * kk < P1 && (h == 0 || l != kk)) {
+            float4 a = h == 0 ? a1 : a2;
+            const size_t o = (size_t)to * nM + c * P1 + l;
+            ff_cadd(a, Lx[o]);
+            a = ff_norm(a);
+            L[o] = a;
+            if (keep) keep[c * P1 + l] = a;
         }
-        for (; k < P1; ++k) {
-            const float4 tq = Tq[k];
-            for (int c = 0; c < 3; ++c) ff_cfma(acc[c], tq, sp[w][c * P1 + k]);
-        }
-    }
-    for (int c = 0; c < 3; ++c)
-        L[((size_t)cell * 3 + c) * P1 + l] =
-            make_double2((double)acc[c].x + (double)acc[c].z, (double)acc[c].y + (double)acc[c].w);
+    };
+    if (up && tid < nM) sp[tid] = L[(size_t)parent[cell] * nM + tid];
+    __syncthreads();
+    if (warp < 3) step(cell, quad[cell], warp, sp, up != 0, sc);
+    if (mask == 0) return;
+    __syncthreads();
+    const int q = warp & 3;
+    if (mask >> q & 1) step(child0[cell] + q, q, warp >> 2, sc, true, nullptr);
 }
 
 // ------------------------------------- stored rows in float-float --
@@ -792,7 +789,7 @@ __device__ __forceinline__ void ff_row_fma(float4 &acc, float4 row, float2 d) {
 static __global__ void __launch_bounds__(kChunk) p2m_rows_ff_kernel(TreeView<double> t, const int *__restrict__ leaves,
                                                                     const double *__restrict__ sb,
                                                                     const double *__restrict__ mb, int use_s,
-                                                                    int use_m, int P1, double2 *__restrict__ M,
+                                                                    int use_m, int P1, float4 *__restrict__ M,
                                                                     const float4 *__restrict__ rows_g,
                                                                     const float4 *__restrict__ rows_f) {
     __shared__ float2 D[kChunk * 6];
@@ -834,12 +831,11 @@ static __global__ void __launch_bounds__(kChunk) p2m_rows_ff_kernel(TreeView<dou
         for (int c = 0; c < 3; ++c) {
             float4 a = part[c * P1 + tid];
             for (int q = 1; q < ngrp; ++q) ff_cadd(a, part[(q * 3 + c) * P1 + tid]);
-            M[((size_t)cell * 3 + c) * P1 + tid] =
-                make_double2((double)a.x + (double)a.z, (double)a.y + (double)a.w);
+            M[((size_t)cell * 3 + c) * P1 + tid] = ff_norm(a);
         }
 }
 
-// Lout[cell] += sum over the cell's list-4 rows (row_off, row_cnt, item as
+// Lout[cell] = sum over the cell's list-4 rows (row_off, row_cnt, item as
 // in p2l_flat_kernel) of rows_g sigma_bar + rows_f mu_bar.
 static __global__ void __launch_bounds__(kChunk) p2l_rows_ff_kernel(TreeView<double> t, const int *__restrict__ cells,
                                                                     const long long *__restrict__ row_off,
@@ -847,7 +843,7 @@ static __global__ void __launch_bounds__(kChunk) p2l_rows_ff_kernel(TreeView<dou
                                                                     const int2 *__restrict__ item,
                                                                     const double *__restrict__ sb,
                                                                     const double *__restrict__ mb, int use_s,
-                                                                    int use_m, int P1, double2 *__restrict__ Lout,
+                                                                    int use_m, int P1, float4 *__restrict__ Lout,
                                                                     const float4 *__restrict__ rows_g,
                                                                     const float4 *__restrict__ rows_f) {
     __shared__ float2 D[kChunk * 6];
@@ -890,10 +886,16 @@ static __global__ void __launch_bounds__(kChunk) p2l_rows_ff_kernel(TreeView<dou
         for (int c = 0; c < 3; ++c) {
             float4 a = part[c * P1 + tid];
             for (int q = 1; q < ngrp; ++q) ff_cadd(a, part[(q * 3 + c) * P1 + tid]);
-            double2 *o = Lout + ((size_t)cell * 3 + c) * P1 + tid;
-            o->x += (double)a.x + (double)a.z;
-            o->y += (double)a.y + (double)a.w;
+            Lout[((size_t)cell * 3 + c) * P1 + tid] = ff_norm(a);
         }
+}
+
+// the FP64 values of float-float expansions
+static __global__ void ff_to_rows_kernel(const float4 *__restrict__ in, double2 *__restrict__ out, size_t n) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const float4 v = in[i];
+        out[i] = make_double2((double)v.x + (double)v.z, (double)v.y + (double)v.w);
+    }
 }
 
 // float-float copies of FP64 complex rows
@@ -922,8 +924,8 @@ inline size_t m2l_ff_smem(int P1) {
 static __global__ void __launch_bounds__(32 * kM2LffWarps) m2l_ff_kernel(TreeView<double> t, const int *__restrict__ cells,
                                                                          int n_cells, int P1,
                                                                          const float4 *__restrict__ base,
-                                                                         const double2 *__restrict__ M,
-                                                                         double2 *__restrict__ Lout) {
+                                                                         const float4 *__restrict__ M,
+                                                                         float4 *__restrict__ Lout) {
     extern __shared__ unsigned char smem_raw[];
     float4 *B = reinterpret_cast<float4 *>(smem_raw);                 // [7][P1][P1]
     float4 *stage = B + 7 * P1 * P1;                                  // [warps][2][3 * 32]
@@ -938,18 +940,18 @@ static __global__ void __launch_bounds__(32 * kM2LffWarps) m2l_ff_kernel(TreeVie
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int ci = blockIdx.x * kM2LffWarps + warp; ci < n_cells; ci += gridDim.x * kM2LffWarps) {
         const int cell = cells[ci];
-        const double mlogw = -t.logw[cell];
+        const float2 mlogw = ff_of(-t.logw[cell]);
         float4 acc[3] = {zero, zero, zero};
-        double acc0[3] = {0.0, 0.0, 0.0};    // the -log(w) Mt_0 term of l = 0, in FP64
+        float2 acc0[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};   // the -log(w) Mt_0 terms
         const int e0 = t.v_ptr[cell], e1 = t.v_ptr[cell + 1];
-        double2 pf[3];
+        float4 pf[3];
         int code = 0;
         auto fetch = [&](int e) {
-            const double2 *ms = M + (size_t)t.v_idx[e] * nM;
+            const float4 *ms = M + (size_t)t.v_idx[e] * nM;
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 const int idx = lane + 32 * j;
-                pf[j] = idx < nM ? ms[idx] : make_double2(0.0, 0.0);
+                pf[j] = idx < nM ? ms[idx] : zero;
             }
             code = t.v_code[e];
         };
@@ -962,15 +964,17 @@ static __global__ void __launch_bounds__(32 * kM2LffWarps) m2l_ff_kernel(TreeVie
             for (int j = 0; j < 3; ++j) {
                 const int idx = lane + 32 * j;
                 if (idx < nM) {
-                    float4 v = ff_rot(ff_from(pf[j]), r * (idx % P1));
+                    float4 v = ff_rot(pf[j], r * (idx % P1));
                     cur[idx] = cj ? ff_conj(v) : v;
                 }
             }
-            const double2 *ms0 = M + (size_t)t.v_idx[e] * nM;
+            __syncwarp();
             if (lane == 0)
 #pragma unroll
-                for (int c = 0; c < 3; ++c) acc0[c] += mlogw * ms0[c * P1].x;    // Mt_0 is real
-            __syncwarp();
+                for (int c = 0; c < 3; ++c) {   // Mt_0 is real
+                    const float4 m0 = cur[c * P1];
+                    ff_fma(acc0[c].x, acc0[c].y, mlogw.x, mlogw.y, m0.x, m0.z);
+                }
             if (e + 1 < e1) fetch(e + 1);
             float4 part[3] = {zero, zero, zero};
             float2 tail[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -1005,10 +1009,11 @@ static __global__ void __launch_bounds__(32 * kM2LffWarps) m2l_ff_kernel(TreeVie
         if (lane < P1)
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                double2 o;
-                o.x = ((double)acc[c].x + (double)acc[c].z) + (lane == 0 ? acc0[c] : 0.0);
-                o.y = (double)acc[c].y + (double)acc[c].w;
-                Lout[((size_t)cell * 3 + c) * P1 + lane] = o;
+                float4 *o = Lout + ((size_t)cell * 3 + c) * P1 + lane;   // onto the list-4 terms
+                float4 a = *o;
+                ff_cadd(a, acc[c]);
+                if (lane == 0) ff_cadd(a, make_float4(acc0[c].x, 0.f, acc0[c].y, 0.f));
+                *o = ff_norm(a);
             }
     }
 }
@@ -1146,33 +1151,6 @@ __global__ void __launch_bounds__(kChunk) p2l_kernel(TreeView<T> t, PS ps, const
 }
 
 // ---------------------------------------------------------------- L2L --
-// One level: L = L_m2l + L2L(parent) (Eq. 73) for the listed cells (the
-// parent term from level 3 on), one warp per cell, lane l holds coefficient l.
-template <typename T>
-__global__ void __launch_bounds__(32 * kLevelWarps) l2l_kernel(TreeView<T> t, const int *__restrict__ cells, int n,
-                                                               int level, int P1,
-                                                               const typename V2<T>::type *__restrict__ tab,
-                                                               const typename V2<T>::type *__restrict__ Lm2l,
-                                                               typename V2<T>::type *__restrict__ L) {
-    using C = typename V2<T>::type;
-    const int idx = blockIdx.x * kLevelWarps + (threadIdx.x >> 5);
-    const int l = threadIdx.x & 31;
-    if (idx >= n || l >= P1) return;
-    const int cell = cells[idx];
-    C acc[3];
-    for (int c = 0; c < 3; ++c) acc[c] = Lm2l[((size_t)cell * 3 + c) * P1 + l];
-    if (level >= 3) {
-        const int par = t.parent[cell], q = t.quad[cell];
-        const C *Tq = tab + ((size_t)q * P1 + l) * P1;
-        const C *src = L + (size_t)par * 3 * P1;
-        for (int k = l; k < P1; ++k) {
-            C tq = Tq[k];
-            for (int c = 0; c < 3; ++c) cfma(acc[c], tq, src[c * P1 + k]);
-        }
-    }
-    for (int c = 0; c < 3; ++c) L[((size_t)cell * 3 + c) * P1 + l] = acc[c];
-}
-
 // Incoming expansion of each listed leaf by the recursion of Eq. 73 along its
 // ancestors: L = Lm2l(a_2) at the level-2 ancestor, then L = Lm2l(a) +
 // L2L(L) for each ancestor a below it and the leaf itself (the level-invariant

@@ -181,12 +181,13 @@ __device__ __noinline__ D3 l2p64(const EvalArgs32 &a, int leaf, double qx, doubl
     D3 h;
     const double iw = 1.0 / a.t64.cw[leaf];
     const double zx = (qx - a.t64.cc[2 * leaf]) * iw, zy = (qy - a.t64.cc[2 * leaf + 1]) * iw;
-    const double2 *Lc = a.L64 + (size_t)leaf * 3 * a.P1;
+    const float4 *Lc = a.L64 + (size_t)leaf * 3 * a.P1;
     for (int ch = 0; ch < 3; ++ch) {
-        double sx = Lc[ch * a.P1 + a.P1 - 1].x, sy = Lc[ch * a.P1 + a.P1 - 1].y;
-        for (int k = a.P1 - 2; k >= 0; --k) {
-            const double nx = sx * zx - sy * zy + Lc[ch * a.P1 + k].x;
-            sy = sx * zy + sy * zx + Lc[ch * a.P1 + k].y;
+        double sx = 0.0, sy = 0.0;
+        for (int k = a.P1 - 1; k >= 0; --k) {
+            const double2 l = ff_value(Lc[ch * a.P1 + k]);
+            const double nx = sx * zx - sy * zy + l.x;
+            sy = sx * zy + sy * zx + l.y;
             sx = nx;
         }
         h.v[ch] = sx * kInv2Pi;
@@ -204,14 +205,15 @@ __device__ __noinline__ D3 m2p64(const EvalArgs32 &a, int src, double qx, double
     const double izx = zx * d, izy = -zy * d;
     const double lz = 0.5 * log(zx * zx + zy * zy) + log(a.t64.cw[src]);
     for (int ch = 0; ch < 3; ++ch) {
-        const double2 *m = a.M64 + ((size_t)src * 3 + ch) * P1;
-        double sx = m[P1 - 1].x / (P1 - 1), sy = m[P1 - 1].y / (P1 - 1);
-        for (int k = P1 - 2; k >= 1; --k) {
-            const double nx = sx * izx - sy * izy + m[k].x / k;
-            sy = sx * izy + sy * izx + m[k].y / k;
+        const float4 *m = a.M64 + ((size_t)src * 3 + ch) * P1;
+        double sx = 0.0, sy = 0.0;
+        for (int k = P1 - 1; k >= 1; --k) {
+            const double2 v = ff_value(m[k]);
+            const double nx = sx * izx - sy * izy + v.x / k;
+            sy = sx * izy + sy * izx + v.y / k;
             sx = nx;
         }
-        h.v[ch] = ((sx * izx - sy * izy) - lz * m[0].x) * kInv2Pi;
+        h.v[ch] = ((sx * izx - sy * izy) - lz * ff_value(m[0]).x) * kInv2Pi;
     }
     return h;
 }
