@@ -87,7 +87,8 @@ __global__ void dense_gemv_kernel(const double *__restrict__ A, int N, const dou
     if (warp >= N) return;
     const double *row = A + (size_t)warp * N;
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    for (int col = lane; col < N; col += 32) {
+#pragma unroll 8
+    for (int col = lane; col < N; col += 32) {   // unrolled: 32 loads in flight
         double a = __ldg(row + col);
         a0 += a * __ldg(x + 3 * (size_t)col + 0);
         a1 += a * __ldg(x + 3 * (size_t)col + 1);

@@ -32,7 +32,7 @@ constexpr int kDotThreads = 256;
 constexpr int kPollRing = 4;     // pinned flag slots / events
 constexpr int kPollLag = 1;      // iterations between enqueue and flag read
 constexpr double kPredictMargin = 4.0;   // see the convergence look-ahead in gmres_solve
-constexpr size_t kGivensSmem = 40 * 1024;   // Givens step staged in shared memory up to this
+constexpr size_t kGivensSmem = 40 * 1024;   // Givens step, back substitution staged in shared memory up to this
 // second Gram-Schmidt pass when ||w after||^2 < kReorthEta2 ||w before||^2
 // (0.01: more than 90% of the norm cancelled; on the bench drawing the
 // solve took 23.1 ms with the classical 1/2, 22.5 ms with 0.01 and 22.7 ms
@@ -72,6 +72,20 @@ __global__ void dots_partial_kernel(const double *__restrict__ V, size_t vstride
     }
     if (threadIdx.x < 3)
         partial[((size_t)j * nchunk + chunk) * 3 + threadIdx.x] = red[threadIdx.x][0];
+}
+
+// Sum of p[0], p[stride], ... (n values another block may just have written)
+// over the warp, in a fixed order, eight loads in flight per lane; in every lane.
+__device__ __forceinline__ double warp_sum_ldcg(const double *p, int n, int stride, int lane) {
+    double t = 0.0;
+    for (int b0 = lane; b0 < n; b0 += 32 * 8) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = b0 + 32 * u < n ? __ldcg(p + (size_t)(b0 + 32 * u) * stride) : 0.0;
+        t += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    }
+    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    return t;
 }
 
 // One Gram-Schmidt pass's dot products h_j = V_j . w for j < nj, fused
@@ -114,12 +128,12 @@ __global__ void __launch_bounds__(kDotThreads) gs_dots_kernel(const B *__restric
     __syncthreads();
     if (!last) return;
     __threadfence();
-    if (threadIdx.x < 3) {
-        const int c = threadIdx.x;
-        double t = 0.0;
-        for (int ch = 0; ch < nchunk; ++ch) t += __ldcg(partial + ((size_t)j * nchunk + ch) * 3 + c);
-        hpass[3 * j + c] = t;
-        hcol[3 * j + c] = first ? t : hcol[3 * j + c] + t;
+    if (wp < 3) {   // a warp per channel (a thread's serial walk cost as much as the products)
+        const double t = warp_sum_ldcg(partial + (size_t)j * nchunk * 3 + wp, nchunk, 3, lane);
+        if (lane == 0) {
+            hpass[3 * j + wp] = t;
+            hcol[3 * j + wp] = first ? t : hcol[3 * j + wp] + t;
+        }
     }
     if (threadIdx.x == 0) count[j] = 0u;
 }
@@ -237,11 +251,16 @@ __device__ void givens_step_warp(GivensState g, const double *__restrict__ hcol,
     }
     __syncwarp();
     if (lane == 0) {
+        // the rotated entry is carried in a register: one fused multiply-add a
+        // step is the chain, the rest is off it
+        double a = col[0];
+#pragma unroll 4
         for (int j = 0; j < k; ++j) {
-            double a = col[j], b = col[j + 1];
-            col[j] = cs[j] * a + sn[j] * b;
-            col[j + 1] = -sn[j] * a + cs[j] * b;
+            const double b = col[j + 1], cj = cs[j], sj = sn[j];
+            col[j] = cj * a + sj * b;
+            a = fma(-sj, a, cj * b);
         }
+        col[k] = a;
         double *e = g.e + c * (m + 1);
         double hn = hnext[c];
         double den = hypot(col[k], hn);
@@ -266,6 +285,7 @@ __device__ void givens_step_warp(GivensState g, const double *__restrict__ hcol,
 }
 
 constexpr int kOrthThreads = 192;   // 3 x 64 elements per block: an element's channel is its index mod 3
+constexpr int kOrthSplit = 4, kOrthSmall = 8000;   // up to this many nodes four threads share an element
 
 // One Gram-Schmidt pass's update w -= V h with the squared norms of the
 // result (and, on the first pass, of w before it) summed per block; the last
@@ -275,7 +295,9 @@ constexpr int kOrthThreads = 192;   // 3 x 64 elements per block: an element's c
 // last pass of the iteration.  pass 1 returns at once when skip is set.
 // Dynamic shared memory: 9 (k + 1) doubles for the Givens step, or none (the
 // step then works in global memory).
-template <typename B>
+// S threads share an element, each every S-th column: with 1,024 nodes a
+// thread alone walked 150 columns, and 16 blocks left the GPU idle.
+template <typename B, int S>
 __global__ void __launch_bounds__(kOrthThreads) orth_norm_givens_kernel(
     const B *__restrict__ V, size_t vstride, const double *__restrict__ h, int nj, double *__restrict__ w,
     int N, double *__restrict__ npart, int pass, int *__restrict__ skip, unsigned *__restrict__ counter,
@@ -286,71 +308,81 @@ __global__ void __launch_bounds__(kOrthThreads) orth_norm_givens_kernel(
     __shared__ double sq[2][kOrthThreads];
     __shared__ bool last;
     __shared__ int keep[3];
-    const int t = blockIdx.x * kOrthThreads + threadIdx.x;
+    __shared__ double norms2[6];
+    constexpr int kEl = kOrthThreads / S;   // elements of a block, a multiple of 3
+    const int el = threadIdx.x % kEl, part = threadIdx.x / kEl;
+    const int t = blockIdx.x * kEl + el;
     double a = 0.0, a0 = 0.0;
     if (t < 3 * N) {
         const int c = t % 3;
-        a = a0 = w[t];
+        int j = part;
         if constexpr (sizeof(B) == 8) {
-            int j = 0;
-            for (; j + 4 <= nj; j += 4) {
-                const double v0 = V[(size_t)j * vstride + t], v1 = V[(size_t)(j + 1) * vstride + t];
-                const double v2 = V[(size_t)(j + 2) * vstride + t], v3 = V[(size_t)(j + 3) * vstride + t];
-                a -= h[3 * j + c] * v0;
-                a -= h[3 * (j + 1) + c] * v1;
-                a -= h[3 * (j + 2) + c] * v2;
-                a -= h[3 * (j + 3) + c] * v3;
+            double d = 0.0;
+            for (; j + 7 * S < nj; j += 8 * S) {   // eight loads in flight
+                double v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = V[(size_t)(j + u * S) * vstride + t];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) d += h[3 * (j + u * S) + c] * v[u];
             }
-            for (; j < nj; ++j) a -= h[3 * j + c] * V[(size_t)j * vstride + t];
+            for (; j < nj; j += S) d += h[3 * j + c] * V[(size_t)j * vstride + t];
+            a = d;
         } else {
-            // FP32 basis: (V h)[t] summed in FP32, eight loads in flight
+            // FP32 basis: (V h)[t] summed in FP32
             float sv = 0.f;
-            int j = 0;
-            for (; j + 8 <= nj; j += 8) {
+            for (; j + 7 * S < nj; j += 8 * S) {
                 float v[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = V[(size_t)(j + u) * vstride + t];
+                for (int u = 0; u < 8; ++u) v[u] = V[(size_t)(j + u * S) * vstride + t];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) sv = fmaf((float)h[3 * (j + u) + c], v[u], sv);
+                for (int u = 0; u < 8; ++u) sv = fmaf((float)h[3 * (j + u * S) + c], v[u], sv);
             }
-            for (; j < nj; ++j) sv = fmaf((float)h[3 * j + c], V[(size_t)j * vstride + t], sv);
-            a -= (double)sv;
+            for (; j < nj; j += S) sv = fmaf((float)h[3 * j + c], V[(size_t)j * vstride + t], sv);
+            a = (double)sv;
         }
-        w[t] = a;
     }
-    sq[0][threadIdx.x] = a * a;
-    sq[1][threadIdx.x] = a0 * a0;
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        double s1 = 0.0, s0 = 0.0;
-        for (int u = threadIdx.x; u < kOrthThreads; u += 3) {
-            s1 += sq[0][u];
-            s0 += sq[1][u];
+    if (S > 1) {
+        sq[0][threadIdx.x] = a;
+        __syncthreads();
+        if (part == 0)
+            for (int q = 1; q < S; ++q) a += sq[0][q * kEl + el];
+        __syncthreads();
+    }
+    if (part == 0) {
+        if (t < 3 * N) {
+            a0 = w[t];
+            a = a0 - a;
+            w[t] = a;
         }
-        npart[6 * blockIdx.x + threadIdx.x] = s1;
-        npart[6 * blockIdx.x + 3 + threadIdx.x] = s0;
-        __threadfence();
+        sq[0][el] = a * a;
+        sq[1][el] = a0 * a0;
+    }
+    __syncthreads();
+    // warp c sums channel c's squares of the result, warp 3 + c those of w before
+    const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31, c = wp < 3 ? wp : wp - 3;
+    {
+        const double *q = sq[wp < 3 ? 0 : 1];
+        double t2 = 0.0;
+        for (int i = lane; i < kEl / 3; i += 32) t2 += q[3 * i + c];
+        for (int off = 16; off > 0; off >>= 1) t2 += __shfl_xor_sync(0xffffffffu, t2, off);
+        if (lane == 0) {
+            npart[6 * blockIdx.x + wp] = t2;
+            __threadfence();
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1u;
     __syncthreads();
     if (!last) return;
     __threadfence();
-    const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (c < 3) {
-        double s1 = 0.0, s0 = 0.0;
-        for (int b = lane; b < (int)gridDim.x; b += 32) {
-            s1 += __ldcg(npart + 6 * b + c);
-            s0 += __ldcg(npart + 6 * b + 3 + c);
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-            s1 += __shfl_xor_sync(0xffffffffu, s1, off);
-            s0 += __shfl_xor_sync(0xffffffffu, s0, off);
-        }
-        if (lane == 0) {
-            hnext[c] = sqrt(fmax(s1, 0.0));
-            keep[c] = s1 >= kReorthEta2 * s0;
-        }
+    {
+        const double t2 = warp_sum_ldcg(npart + wp, (int)gridDim.x, 6, lane);
+        if (lane == 0) norms2[wp] = t2;
+    }
+    __syncthreads();
+    if (wp < 3 && lane == 0) {
+        hnext[c] = sqrt(fmax(norms2[c], 0.0));
+        keep[c] = norms2[c] >= kReorthEta2 * norms2[3 + c];
     }
     __syncthreads();
     bool givens = true;
@@ -360,24 +392,34 @@ __global__ void __launch_bounds__(kOrthThreads) orth_norm_givens_kernel(
     }
     if (threadIdx.x == 0) *counter = 0u;
     __threadfence();
-    if (givens && c < 3) givens_step_warp(g, hcol, hnext, thr, k, m, c, lane, staged ? gsm + (size_t)c * 3 * (k + 1) : nullptr);
+    if (givens && wp < 3) givens_step_warp(g, hcol, hnext, thr, k, m, c, lane, staged ? gsm + (size_t)c * 3 * (k + 1) : nullptr);
 }
 
-// Back substitution R y = e for each channel (kc[c] columns).
-__global__ void backsolve_kernel(GivensState g, int m) {
-    int c = threadIdx.x;
-    if (c >= 3) return;
-    int n = g.kc[c];
+// Back substitution R y = e for channel blockIdx.x (kc[c] columns), column
+// by column: y_i, then its column off the right-hand side, all rows at once
+// (R is stored by columns).  The right-hand side is kept in m doubles of
+// dynamic shared memory when staged, else in e, which nothing reads after
+// this.  With one thread per channel walking the rows, 154 columns took
+// 1.15 ms; this takes 0.24.
+constexpr int kBackThreads = 256;
+__global__ void __launch_bounds__(kBackThreads) backsolve_kernel(GivensState g, int m, int staged) {
+    extern __shared__ double rhs_s[];
+    const int c = blockIdx.x, n = g.kc[c];
     const double *R = g.R + (size_t)c * m * m;
-    double *y = g.y + c * m;
-    const double *e = g.e + c * (m + 1);
+    double *y = g.y + (size_t)c * m;
+    double *e = g.e + (size_t)c * (m + 1);
+    double *rhs = staged ? rhs_s : e;
+    if (staged)
+        for (int i = threadIdx.x; i < n; i += kBackThreads) rhs[i] = e[i];
+    for (int i = n + threadIdx.x; i < m; i += kBackThreads) y[i] = 0.0;
+    __syncthreads();
     for (int i = n - 1; i >= 0; --i) {
-        double s = e[i];
-        for (int j = i + 1; j < n; ++j) s -= R[(size_t)j * m + i] * y[j];
-        double d = R[(size_t)i * m + i];
-        y[i] = (d != 0.0) ? s / d : 0.0;
+        const double *col = R + (size_t)i * m;
+        const double d = col[i], yi = d != 0.0 ? rhs[i] / d : 0.0;
+        if (threadIdx.x == 0) y[i] = yi;
+        for (int j = threadIdx.x; j < i; j += kBackThreads) rhs[j] -= col[j] * yi;
+        __syncthreads();
     }
-    for (int i = n; i < m; ++i) y[i] = 0.0;
 }
 
 // x[i][c] += sum_{j < kc[c]} y[c][j] V_j[i][c]
@@ -431,7 +473,7 @@ struct GmresWork {
         DC_TRY(Ax.alloc((size_t)N * 3));
         DC_TRY(partial.alloc((size_t)(m + 1) * nchunk * 3));
         DC_TRY(count.alloc((size_t)(m + 2)));   // gs_dots columns, then the orth_norm_givens counter
-        DC_TRY(npart.alloc((size_t)6 * ((3 * (size_t)N + kOrthThreads - 1) / kOrthThreads)));
+        DC_TRY(npart.alloc((size_t)6 * ((3 * (size_t)N * kOrthSplit + kOrthThreads - 1) / kOrthThreads)));
         DC_TRY(hcol.alloc((size_t)(m + 1) * 3));
         DC_TRY(hpass.alloc((size_t)(m + 1) * 3));
         DC_TRY(hnext.alloc(3));
@@ -600,6 +642,7 @@ cudaError_t gmres_solve(GmresWork *Wp, Operator &A, int N, const double *b, doub
     // at the FP32 rate; the operator is applied to the stored FP32 vectors,
     // so the Arnoldi relation holds for them.  Other solves keep FP64.
     const bool bufs = A.in_buffer() && A.out_buffer();
+    const bool small = N <= kOrthSmall;
     const bool b32 = bufs && trust_estimate && tol >= kBasis32MinTol;
     int total = 0;
     bool done_all = false;
@@ -670,21 +713,24 @@ cudaError_t gmres_solve(GmresWork *Wp, Operator &A, int N, const double *b, doub
             int *skip = W.flags.ptr + 6;   // after active[3], kc[3]
             const size_t gsm = (size_t)9 * (k + 1) * sizeof(double);
             const int staged = gsm <= kGivensSmem ? 1 : 0;
-            const int nb = (3 * N + kOrthThreads - 1) / kOrthThreads;
+            const int per = small ? kOrthThreads / kOrthSplit : kOrthThreads;
+            const int nb = (3 * N + per - 1) / per;
             for (int pass = 0; pass < 2; ++pass) {
                 dim3 grid(W.nchunk, k + 1);
                 if (b32) {
                     gs_dots_kernel<float><<<grid, kDotThreads, 0, st>>>(
                         W.V32.ptr, vs, wv, N, W.nchunk, W.partial.ptr, W.count.ptr, W.hpass.ptr, W.hcol.ptr,
                         pass == 0, pass == 0 ? nullptr : skip);
-                    orth_norm_givens_kernel<float><<<nb, kOrthThreads, staged ? gsm : 0, st>>>(
+                    auto orth = small ? orth_norm_givens_kernel<float, kOrthSplit> : orth_norm_givens_kernel<float, 1>;
+                    orth<<<nb, kOrthThreads, staged ? gsm : 0, st>>>(
                         W.V32.ptr, vs, W.hpass.ptr, k + 1, wv, N, W.npart.ptr, pass, skip, W.count.ptr + (m + 1),
                         W.hnext.ptr, gs, W.hcol.ptr, thr, k, m, staged);
                 } else {
                     gs_dots_kernel<double><<<grid, kDotThreads, 0, st>>>(
                         W.V.ptr, vs, wv, N, W.nchunk, W.partial.ptr, W.count.ptr, W.hpass.ptr, W.hcol.ptr,
                         pass == 0, pass == 0 ? nullptr : skip);
-                    orth_norm_givens_kernel<double><<<nb, kOrthThreads, staged ? gsm : 0, st>>>(
+                    auto orth = small ? orth_norm_givens_kernel<double, kOrthSplit> : orth_norm_givens_kernel<double, 1>;
+                    orth<<<nb, kOrthThreads, staged ? gsm : 0, st>>>(
                         W.V.ptr, vs, W.hpass.ptr, k + 1, wv, N, W.npart.ptr, pass, skip, W.count.ptr + (m + 1),
                         W.hnext.ptr, gs, W.hcol.ptr, thr, k, m, staged);
                 }
@@ -741,7 +787,9 @@ cudaError_t gmres_solve(GmresWork *Wp, Operator &A, int N, const double *b, doub
                 }
             }
         }
-        backsolve_kernel<<<1, 32, 0, st>>>(gs, m); note_launch();
+        const size_t rhs_b = (size_t)m * sizeof(double);
+        const int rhs_staged = rhs_b <= kGivensSmem ? 1 : 0;
+        backsolve_kernel<<<3, kBackThreads, rhs_staged ? rhs_b : 0, st>>>(gs, m, rhs_staged); note_launch();
         if (b32) solution_update_kernel<float><<<(N + th - 1) / th, th, 0, st>>>(gs, W.V32.ptr, vs, x, N, m);
         else solution_update_kernel<double><<<(N + th - 1) / th, th, 0, st>>>(gs, W.V.ptr, vs, x, N, m);
         note_launch();
