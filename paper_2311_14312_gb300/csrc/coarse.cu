@@ -487,6 +487,180 @@ __global__ void __launch_bounds__(kMonoThreads) monopole_kernel(const float2 *__
     }
 }
 
+// ---- the monopoles by clusters -----------------------------------------
+// From kTreePanels panels up the sum over all panels at every node (N P
+// logarithms: 890 M for 7,459 panels, 313 us, 60% of the rate of the special
+// function unit) is taken over a binary tree of clusters instead, whose
+// leaves are kLeafPanels panels consecutive in Morton order.  For a leaf's
+// nodes a cluster whose circle is at least kClusterSep of its radii away
+// contributes by its moments up to order kOrder about its centre, the others
+// panel by panel.  An entry's terms are summed by themselves before they join
+// the node's sum.  At order 8 the series' remainder, 0.4^9 / 9 = 3e-5 of a far
+// term at the nearest distance, is below rounding in the result: against the
+// same sums in FP64, M v of a random v is off by 6.9e-7 (the direct sum:
+// 9.6e-7), of a constant by 4.1e-4 of what is left after cancellation (2.0e-3).
+// One application of M takes 256 us instead of 474 (2,173 panels: 62 and 72),
+// that drawing's solve 32.7 ms instead of 40.3.  The lists are made on the host with the plan and cut into kSplit parts:
+// with one block to a leaf the longest lists set the time (at order 5 the
+// solve took 35.5, 32.3 and 31.9 ms with 1, 4 and 8 parts).
+constexpr int kTreePanels = 1024, kLeafPanels = 8, kOrder = 8;
+constexpr double kClusterSep = 2.5;
+// a node's moments: (M_0 of the channels, -), then per order (re, im of
+// channels 0, 1) and (re, im of channel 2, -, -)
+constexpr int kMomentRows = 1 + 2 * kOrder;       // float4
+constexpr int kTreeThreads = 128, kTreeStage = 16;
+
+// Moments of node nodes[blockIdx.x]'s panels about its centre, in its radius:
+// M_0 = sum k, M_n = -(2 / (n ln 2)) sum k z^n (for sum k lg2 |q - c|^2 = M_0
+// lg2 |d|^2 + Re sum M_n (rad / d)^n).
+__global__ void __launch_bounds__(kTreeThreads) cluster_moments_kernel(const int *__restrict__ nodes,
+                                                                       const float4 *__restrict__ geo,
+                                                                       const int2 *__restrict__ range,
+                                                                       const int *__restrict__ mo,
+                                                                       const float4 *__restrict__ pan,
+                                                                       const float *__restrict__ pan2,
+                                                                       float4 *__restrict__ mom) {
+    constexpr int kVals = 3 + 6 * kOrder;
+    __shared__ float red[kTreeThreads / 32][kVals];
+    const int b = nodes[blockIdx.x], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float4 gm = geo[b];   // centre, radius, 1 / radius
+    const int2 r = range[b];
+    float m[kVals];
+#pragma unroll
+    for (int i = 0; i < kVals; ++i) m[i] = 0.f;
+    for (int p = r.x + threadIdx.x; p < r.y; p += kTreeThreads) {
+        const int j = mo[p];
+        const float4 a = pan[j];
+        const float k[3] = {a.z, a.w, pan2[j]};
+        const float zx = (a.x - gm.x) * gm.w, zy = (a.y - gm.y) * gm.w;
+        float wx = zx, wy = zy;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) m[c] += k[c];
+#pragma unroll
+        for (int n = 0; n < kOrder; ++n) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                m[3 + 6 * n + 2 * c] += k[c] * wx;
+                m[4 + 6 * n + 2 * c] += k[c] * wy;
+            }
+            const float t = wx * zx - wy * zy;
+            wy = wx * zy + wy * zx;
+            wx = t;
+        }
+    }
+    const int warps = min(kTreeThreads / 32, (r.y - r.x + 31) / 32);   // those that had panels
+    if (warp < warps)
+#pragma unroll
+        for (int i = 0; i < kVals; ++i) {
+            for (int o = 16; o > 0; o >>= 1) m[i] += __shfl_xor_sync(0xffffffffu, m[i], o);
+            if (lane == 0) red[warp][i] = m[i];
+        }
+    __syncthreads();
+    if (threadIdx.x < kVals) {
+        const int i = threadIdx.x;
+        float t = red[0][i];
+        for (int w = 1; w < warps; ++w) t += red[w][i];
+        float *o = reinterpret_cast<float *>(mom + (size_t)b * kMomentRows);
+        if (i < 3) {
+            o[i] = t;
+        } else {
+            const int n = (i - 3) / 6, q = (i - 3) % 6;
+            o[4 + 8 * n + q] = t * (-2.885390082f / (n + 1));
+        }
+    }
+}
+
+// part[blockIdx.y][a] at the nodes a of leaf blockIdx.x: every gridDim.y-th
+// entry of its far list (by moments) and of its near list (by panels)
+__global__ void __launch_bounds__(kTreeThreads) cluster_eval_kernel(const float2 *__restrict__ q32, const float4 *__restrict__ geo,
+                                                                    const int2 *__restrict__ range, const int *__restrict__ mo,
+                                                                    const int2 *__restrict__ fptr, const int *__restrict__ list,
+                                                                    const float4 *__restrict__ pan, const float *__restrict__ pan2,
+                                                                    const float4 *__restrict__ mom, int g, int N,
+                                                                    float *__restrict__ part) {
+    __shared__ float4 sg[kTreeStage];
+    __shared__ float4 sm[kTreeStage][kMomentRows];
+    __shared__ float4 sp[kTreeStage * kLeafPanels];
+    __shared__ float sp2[kTreeStage * kLeafPanels];
+    const int leaf = blockIdx.x, S = gridDim.y, first = range[leaf].x;
+    const int nodes = (range[leaf].y - first) * g;
+    // far entries at list[fptr.x ..), near ones at [fptr.y .. next fptr.x)
+    const int f0 = fptr[leaf].x, f1 = fptr[leaf].y, n1 = fptr[leaf + 1].x;
+    for (int base = 0; base < nodes; base += kTreeThreads) {
+        const int u = base + threadIdx.x, pu = min(u, nodes - 1);
+        const int a = mo[first + pu / g] * g + pu % g;
+        const float2 q = q32[a];
+        float t0 = 0.f, t1 = 0.f, t2 = 0.f;
+        for (int e = f0 + blockIdx.y; e < f1; e += S * kTreeStage) {
+            const int cnt = min(kTreeStage, (f1 - e + S - 1) / S);
+            __syncthreads();
+            for (int i = threadIdx.x; i < cnt * kMomentRows; i += kTreeThreads) {
+                const int w = i / kMomentRows, r = i - w * kMomentRows;
+                sm[w][r] = mom[(size_t)list[e + w * S] * kMomentRows + r];
+            }
+            if (threadIdx.x < cnt) sg[threadIdx.x] = geo[list[e + threadIdx.x * S]];
+            __syncthreads();
+#pragma unroll 2
+            for (int w = 0; w < cnt; ++w) {
+                const float4 gm = sg[w], m0 = sm[w][0];
+                const float dx = q.x - gm.x, dy = q.y - gm.y, r2 = dx * dx + dy * dy;
+                const float lg = __log2f(r2), ir = __fdividef(gm.z, r2);
+                const float vx = dx * ir, vy = -dy * ir;   // rad / d
+                float wx = vx, wy = vy;
+                float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+#pragma unroll
+                for (int n = 0; n < kOrder; ++n) {
+                    const float4 x = sm[w][1 + 2 * n];
+                    const float2 y = *reinterpret_cast<const float2 *>(&sm[w][2 + 2 * n]);
+                    s0 = fmaf(x.x, wx, fmaf(-x.y, wy, s0));
+                    s1 = fmaf(x.z, wx, fmaf(-x.w, wy, s1));
+                    s2 = fmaf(y.x, wx, fmaf(-y.y, wy, s2));
+                    const float s = wx * vx - wy * vy;
+                    wy = wx * vy + wy * vx;
+                    wx = s;
+                }
+                t0 += fmaf(lg, m0.x, s0);
+                t1 += fmaf(lg, m0.y, s1);
+                t2 += fmaf(lg, m0.z, s2);
+            }
+        }
+        for (int e = f1 + blockIdx.y; e < n1; e += S * kTreeStage) {
+            const int cnt = min(kTreeStage, (n1 - e + S - 1) / S);
+            __syncthreads();
+            for (int i = threadIdx.x; i < cnt * kLeafPanels; i += kTreeThreads) {
+                const int2 r = range[list[e + (i / kLeafPanels) * S]];
+                const int p = r.x + i % kLeafPanels;
+                const int j = mo[min(p, r.y - 1)];
+                const float4 v = pan[j];
+                const bool in = p < r.y;   // the last leaf may be short
+                sp[i] = make_float4(v.x, v.y, in ? v.z : 0.f, in ? v.w : 0.f);
+                sp2[i] = in ? pan2[j] : 0.f;
+            }
+            __syncthreads();
+            for (int w = 0; w < cnt; ++w) {
+                float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+#pragma unroll
+                for (int i = w * kLeafPanels; i < (w + 1) * kLeafPanels; ++i) {
+                    const float4 p = sp[i];
+                    const float k = mono_lg2(q, make_float2(p.x, p.y));
+                    s0 = fmaf(k, p.z, s0);
+                    s1 = fmaf(k, p.w, s1);
+                    s2 = fmaf(k, sp2[i], s2);
+                }
+                t0 += s0;
+                t1 += s1;
+                t2 += s2;
+            }
+        }
+        if (u < nodes) {
+            float *o = part + ((size_t)blockIdx.y * N + a) * 3;
+            o[0] = t0;
+            o[1] = t1;
+            o[2] = t2;
+        }
+    }
+}
+
 // Per panel i (one block): r = v - A~ P y at its nodes (the monopole parts,
 // added in part order, plus the near-pair corrections), w = P y + B r with
 // B_i the panel's inverse self-interaction block, written when w is given,
@@ -580,6 +754,36 @@ __global__ void inverse_check_kernel(const float *__restrict__ Ai, const float *
 
 }  // namespace
 
+namespace {
+// the panels in the Morton order of their centroids (16 bits per axis over
+// the centroids' box, ties by panel index)
+std::vector<int> morton_order(const std::vector<double> &cen) {
+    const int P = int(cen.size() / 2);
+    double lo[2] = {cen[0], cen[1]}, hi[2] = {cen[0], cen[1]};
+    for (int j = 0; j < P; ++j)
+        for (int d = 0; d < 2; ++d) {
+            lo[d] = std::min(lo[d], cen[2 * j + d]);
+            hi[d] = std::max(hi[d], cen[2 * j + d]);
+        }
+    std::vector<unsigned long long> key(P);
+    for (int j = 0; j < P; ++j) {
+        unsigned q[2];
+        for (int d = 0; d < 2; ++d) {
+            const double ext = hi[d] - lo[d];
+            const double f = ext > 0.0 ? (cen[2 * j + d] - lo[d]) / ext : 0.0;
+            q[d] = (unsigned)std::min(65535.0, std::floor(f * 65536.0));
+        }
+        unsigned long long k = 0;
+        for (int b = 15; b >= 0; --b) k = (k << 2) | (((q[1] >> b) & 1u) << 1) | ((q[0] >> b) & 1u);
+        key[j] = (k << 32) | (unsigned long long)j;
+    }
+    std::vector<int> perm(P);
+    for (int j = 0; j < P; ++j) perm[j] = j;
+    std::sort(perm.begin(), perm.end(), [&](int a, int b) { return key[a] < key[b]; });
+    return perm;
+}
+}  // namespace
+
 void TwoLevel::plan(const Geometry &G, int max_coarse) {
     ready_ = false;
     planned_ = false;
@@ -628,26 +832,7 @@ void TwoLevel::plan(const Geometry &G, int max_coarse) {
         for (int j = 0; j < P; ++j) perm[j] = agg_of[j] = j;
     } else {
         K_ = (P + (maxc - kGJ) - 1) / (maxc - kGJ);
-        double lo[2] = {cen[0], cen[1]}, hi[2] = {cen[0], cen[1]};
-        for (int j = 0; j < P; ++j)
-            for (int d = 0; d < 2; ++d) {
-                lo[d] = std::min(lo[d], cen[2 * j + d]);
-                hi[d] = std::max(hi[d], cen[2 * j + d]);
-            }
-        std::vector<unsigned long long> key(P);
-        for (int j = 0; j < P; ++j) {
-            unsigned q[2];
-            for (int d = 0; d < 2; ++d) {
-                const double ext = hi[d] - lo[d];
-                const double f = ext > 0.0 ? (cen[2 * j + d] - lo[d]) / ext : 0.0;
-                q[d] = (unsigned)std::min(65535.0, std::floor(f * 65536.0));
-            }
-            unsigned long long k = 0;
-            for (int b = 15; b >= 0; --b) k = (k << 2) | (((q[1] >> b) & 1u) << 1) | ((q[0] >> b) & 1u);
-            key[j] = (k << 32) | (unsigned long long)j;
-        }
-        for (int j = 0; j < P; ++j) perm[j] = j;
-        std::sort(perm.begin(), perm.end(), [&](int a, int b) { return key[a] < key[b]; });
+        perm = morton_order(cen);
     }
     for (int u = 0; u < P; ++u) {
         if (u % K_ == 0) pagg.push_back(u);
@@ -689,7 +874,91 @@ void TwoLevel::plan(const Geometry &G, int max_coarse) {
         }
         nptr[P] = int(pairs.size());
     }
+    n_leaves_ = 0;
+    h_geo_.clear();
+    h_far_.clear();
+    if (K_ == 1 && P >= kTreePanels) plan_clusters(cen, G);
     planned_ = true;
+}
+
+// The cluster tree over the panels and every leaf's lists.
+void TwoLevel::plan_clusters(const std::vector<double> &cen, const Geometry &G) {
+    const int P = P_, g = g_;
+    h_mo_ = morton_order(cen);
+    struct Node {
+        int lo, hi, child, nchild;
+        double x, y, r;
+    };
+    std::vector<Node> nd;
+    auto add = [&](int lo, int hi, int child, int nchild) {
+        double bx0 = 1e300, by0 = 1e300, bx1 = -1e300, by1 = -1e300, r2 = 0.0;
+        for (int p = lo; p < hi; ++p) {
+            const double *c = &cen[2 * (size_t)h_mo_[p]];
+            bx0 = std::min(bx0, c[0]);
+            bx1 = std::max(bx1, c[0]);
+            by0 = std::min(by0, c[1]);
+            by1 = std::max(by1, c[1]);
+        }
+        const double x = (float)(0.5 * (bx0 + bx1)), y = (float)(0.5 * (by0 + by1));
+        for (int p = lo; p < hi; ++p) {
+            const double *c = &cen[2 * (size_t)h_mo_[p]];
+            r2 = std::max(r2, (c[0] - x) * (c[0] - x) + (c[1] - y) * (c[1] - y));
+        }
+        nd.push_back({lo, hi, child, nchild, x, y, std::sqrt(r2)});
+    };
+    for (int lo = 0; lo < P; lo += kLeafPanels) add(lo, std::min(P, lo + kLeafPanels), -1, 0);
+    n_leaves_ = int(nd.size());
+    int lev0 = 0, lev1 = n_leaves_;
+    while (lev1 - lev0 > 1) {
+        for (int i = lev0; i < lev1; i += 2) {
+            const int n = std::min(2, lev1 - i);
+            add(nd[i].lo, nd[i + n - 1].hi, i, n);
+        }
+        lev0 = lev1;
+        lev1 = int(nd.size());
+    }
+    h_fptr_.assign(n_leaves_ + 1, make_int2(0, 0));
+    h_list_.clear();
+    std::vector<int> near, stack;
+    for (int t = 0; t < n_leaves_; ++t) {
+        // the circle of the leaf's nodes about its centre
+        double rt = 0.0;
+        for (int p = nd[t].lo; p < nd[t].hi; ++p)
+            for (int m = 0; m < g; ++m) {
+                const double *q = &G.node_xy[2 * ((size_t)h_mo_[p] * g + m)];
+                rt = std::max(rt, std::hypot(q[0] - nd[t].x, q[1] - nd[t].y));
+            }
+        h_fptr_[t].x = int(h_list_.size());
+        near.clear();
+        stack.assign(1, int(nd.size()) - 1);
+        while (!stack.empty()) {
+            const int b = stack.back();
+            stack.pop_back();
+            const Node &n = nd[b];
+            const double d = std::hypot(n.x - nd[t].x, n.y - nd[t].y) - rt;
+            if (d >= kClusterSep * n.r && d > 0.0) h_list_.push_back(b);
+            else if (n.child < 0) near.push_back(b);
+            else
+                for (int q = 0; q < n.nchild; ++q) stack.push_back(n.child + q);
+        }
+        h_fptr_[t].y = int(h_list_.size());
+        h_list_.insert(h_list_.end(), near.begin(), near.end());
+    }
+    h_fptr_[n_leaves_] = make_int2(int(h_list_.size()), int(h_list_.size()));
+    // the nodes some list takes by its moments
+    std::vector<char> used(nd.size(), 0);
+    for (int t = 0; t < n_leaves_; ++t)
+        for (int e = h_fptr_[t].x; e < h_fptr_[t].y; ++e) used[h_list_[e]] = 1;
+    h_far_.clear();
+    for (size_t b = nd.size(); b-- > 0;)   // the large ones first
+        if (used[b]) h_far_.push_back(int(b));
+    h_geo_.resize(nd.size());
+    h_range_.resize(nd.size());
+    for (size_t b = 0; b < nd.size(); ++b) {
+        const double r = std::max(nd[b].r, 1e-12);   // one panel, or panels at one point
+        h_geo_[b] = make_float4((float)nd[b].x, (float)nd[b].y, (float)r, (float)(1.0 / r));
+        h_range_[b] = make_int2(nd[b].lo, nd[b].hi);
+    }
 }
 
 cudaError_t TwoLevel::launch(const DevGeom &D, cudaStream_t st) {
@@ -714,6 +983,15 @@ cudaError_t TwoLevel::launch(const DevGeom &D, cudaStream_t st) {
     if (K_ > 1 && ((e = up(pagg_, h_pagg_)) != cudaSuccess || (e = up(agg_of_, h_agg_of_)) != cudaSuccess ||
                    (e = up(perm_, h_perm_)) != cudaSuccess))
         return e;
+    n_nodes_ = int(h_geo_.size());
+    n_far_ = int(h_far_.size());
+    if (n_leaves_ > 0) {
+        if ((e = up(mo_, h_mo_)) != cudaSuccess || (e = up(list_, h_list_)) != cudaSuccess ||
+            (e = up(fptr_, h_fptr_)) != cudaSuccess || (e = up(range_, h_range_)) != cudaSuccess ||
+            (e = up(geo_, h_geo_)) != cudaSuccess || (e = up(far_, h_far_)) != cudaSuccess ||
+            (e = mom_.alloc((size_t)n_nodes_ * kMomentRows)) != cudaSuccess)
+            return e;
+    }
     if ((e = corr_.alloc(n_pairs * (size_t)g)) != cudaSuccess ||
         (e = Ainv_.alloc((size_t)n_pad_ * n_pad_)) != cudaSuccess || (e = s_.alloc(3 * (size_t)P)) != cudaSuccess ||
         (e = y_.alloc(3 * (size_t)P)) != cudaSuccess || (e = pan_.alloc((size_t)P)) != cudaSuccess || (e = pan2_.alloc((size_t)P)) != cudaSuccess ||
@@ -766,6 +1044,12 @@ cudaError_t TwoLevel::launch(const DevGeom &D, cudaStream_t st) {
     std::vector<float2>().swap(h_q32_);
     std::vector<float>().swap(h_pl32_);
     std::vector<int2>().swap(h_pairs_);
+    std::vector<int2>().swap(h_fptr_);
+    std::vector<int2>().swap(h_range_);
+    std::vector<float4>().swap(h_geo_);
+    std::vector<int>().swap(h_mo_);
+    std::vector<int>().swap(h_list_);
+    std::vector<int>().swap(h_far_);
     std::vector<int>().swap(h_nptr_);
     std::vector<int>().swap(h_pagg_);
     std::vector<int>().swap(h_perm_);
@@ -805,11 +1089,21 @@ cudaError_t TwoLevel::apply(const double *inv, const double *v, double *w, cudaS
     restrict_kernel<<<(3 * P + 255) / 256, 256, 0, st>>>(v, P, g, s_.ptr);
     coarse_solve_kernel<<<(P + kSolveRows - 1) / kSolveRows, 32 * kSolveRows, 0, st>>>(
         Ainv_.ptr, n_pad_, P, s_.ptr, plen32_.ptr, c32_.ptr, y_.ptr, pan_.ptr, pan2_.ptr);
-    const int per_block = kMonoThreads * kMonoNodes;
-    monopole_kernel<<<dim3((N + per_block - 1) / per_block, kSplit), kMonoThreads, 0, st>>>(q32_.ptr, pan_.ptr,
-                                                                                         pan2_.ptr, P, N, part_.ptr);
-    panel_apply_kernel<<<P, kPanelThreads, 0, st>>>(part_.ptr, N, g, s, nptr_.ptr, pairs_.ptr, corr_.ptr, y_.ptr, v,
-                                                    inv, w, lam, sv, nullptr, nullptr);
+    if (n_leaves_ > 0) {
+        if (n_far_ > 0) {
+            cluster_moments_kernel<<<n_far_, kTreeThreads, 0, st>>>(far_.ptr, geo_.ptr, range_.ptr, mo_.ptr, pan_.ptr, pan2_.ptr,
+                                                                    mom_.ptr);
+            note_launch();
+        }
+        cluster_eval_kernel<<<dim3(n_leaves_, kSplit), kTreeThreads, 0, st>>>(
+            q32_.ptr, geo_.ptr, range_.ptr, mo_.ptr, fptr_.ptr, list_.ptr, pan_.ptr, pan2_.ptr, mom_.ptr, g, N, part_.ptr);
+    } else {
+        const int per_block = kMonoThreads * kMonoNodes;
+        monopole_kernel<<<dim3((N + per_block - 1) / per_block, kSplit), kMonoThreads, 0, st>>>(
+            q32_.ptr, pan_.ptr, pan2_.ptr, P, N, part_.ptr);
+    }
+    panel_apply_kernel<<<P, kPanelThreads, 0, st>>>(part_.ptr, N, g, s, nptr_.ptr, pairs_.ptr, corr_.ptr, y_.ptr,
+                                                    v, inv, w, lam, sv, nullptr, nullptr);
     note_launch(4);
     return cudaGetLastError();
 }

@@ -305,6 +305,16 @@ private:
     std::vector<float> h_pl32_;
     std::vector<int> h_pagg_, h_perm_, h_agg_of_, h_nptr_;
     std::vector<int2> h_pairs_;
+    // the cluster tree of the monopole sums (n_leaves_ = 0: summed directly)
+    void plan_clusters(const std::vector<double> &cen, const Geometry &G);
+    int n_leaves_ = 0, n_nodes_ = 0, n_far_ = 0;
+    std::vector<int> h_mo_, h_list_, h_far_;
+    std::vector<int2> h_fptr_, h_range_;
+    std::vector<float4> h_geo_;
+    DevBuf<int> mo_, list_, far_;   // panels in Morton order; lists of node numbers; nodes with moments
+    DevBuf<int2> fptr_, range_;     // per leaf: first far and first near entry; per node: its panels in mo_
+    DevBuf<float4> geo_;            // per node: centre, radius, 1 / radius
+    DevBuf<float4> mom_;            // per node: moments
     // launch() to finish(): the coarse matrix before inversion, the check's
     // row errors and its bad-pivot flag
     DevBuf<float> Ac_, gj_tmp_;
