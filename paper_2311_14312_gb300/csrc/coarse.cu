@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "dc_internal.h"
+#include "ffmath.cuh"
 #include "ffarith.cuh"
 #include "segint.cuh"
 
@@ -363,7 +364,7 @@ __device__ __forceinline__ void dot2_step(float &hi, float &lo, float w, float2 
     lo += se + pe + w * x.y;
 }
 
-// y = Ac^-1 s (fixed-order reduction); pan[j] = (c_j, k l_j y_j for
+// y = Ac^-1 s (fixed-order reduction), also as (hi, lo) floats; pan[j] = (c_j, k l_j y_j for
 // channels 0, 1), pan2[j] = k l_j y_j for channel 2, k = kMonoLog2 (FP32).
 // One warp per row, kSolveRows rows per block: the vector s is staged in
 // shared memory kSolveCols columns at a time and serves all of the block's
@@ -375,6 +376,7 @@ __global__ void __launch_bounds__(32 * kSolveRows) coarse_solve_kernel(const flo
                                                                        const float *__restrict__ plen32,
                                                                        const float2 *__restrict__ c32,
                                                                        double *__restrict__ y,
+                                                                       float2 *__restrict__ yff,
                                                                        float4 *__restrict__ pan,
                                                                        float *__restrict__ pan2) {
     __shared__ float2 ss[3 * kSolveCols];
@@ -416,6 +418,9 @@ __global__ void __launch_bounds__(32 * kSolveRows) coarse_solve_kernel(const flo
         y[3 * i + 0] = a0;
         y[3 * i + 1] = a1;
         y[3 * i + 2] = a2;
+        yff[3 * i + 0] = ff::from(a0);
+        yff[3 * i + 1] = ff::from(a1);
+        yff[3 * i + 2] = ff::from(a2);
         const float k = kMonoLog2 * plen32[i];
         const float2 c = c32[i];
         pan[i] = make_float4(c.x, c.y, k * (float)a0, k * (float)a1);
@@ -499,11 +504,12 @@ __global__ void __launch_bounds__(kMonoThreads) monopole_kernel(const float2 *__
 // term at the nearest distance, is below rounding in the result: against the
 // same sums in FP64, M v of a random v is off by 6.9e-7 (the direct sum:
 // 9.6e-7), of a constant by 4.1e-4 of what is left after cancellation (2.0e-3).
-// One application of M takes 256 us instead of 474 (2,173 panels: 62 and 72),
-// that drawing's solve 32.7 ms instead of 40.3.  The lists are made on the host with the plan and cut into kSplit parts:
+// One application of M took 256 us instead of 474 (2,173 panels: 62 and 72;
+// 1,750: 56 and 55; 1,010: 40 and 36), that drawing's solve 32.7 ms instead of
+// 40.3.  The lists are made on the host with the plan and cut into kSplit parts:
 // with one block to a leaf the longest lists set the time (at order 5 the
 // solve took 35.5, 32.3 and 31.9 ms with 1, 4 and 8 parts).
-constexpr int kTreePanels = 1024, kLeafPanels = 8, kOrder = 8;
+constexpr int kTreePanels = 2048, kLeafPanels = 8, kOrder = 8;
 constexpr double kClusterSep = 2.5;
 // a node's moments: (M_0 of the channels, -), then per order (re, im of
 // channels 0, 1) and (re, im of channel 2, -, -)
@@ -661,65 +667,86 @@ __global__ void __launch_bounds__(kTreeThreads) cluster_eval_kernel(const float2
     }
 }
 
+// b[i] = a[i] as (hi, lo) floats
+__global__ void to_ff_kernel(const double *__restrict__ a, float2 *__restrict__ b, size_t n) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        b[i] = ff::from(a[i]);
+}
+
 // Per panel i (one block): r = v - A~ P y at its nodes (the monopole parts,
 // added in part order, plus the near-pair corrections), w = P y + B r with
 // B_i the panel's inverse self-interaction block, written when w is given,
-// and, when lam is given, sigma_bar = Lambda w for the panel's s segments in
-// float-float (w converted to hi/lo pairs once, Lambda stored as hi/lo
-// floats), rounded to FP32.
+// and, when lam is given, sigma_bar = Lambda w for the panel's s segments,
+// rounded to FP32.  All of it in float-float: in FP64 the residual and the
+// block product held the FP64 pipe for about 1,000 cycles a panel.  B is
+// staged by the whole block while the first threads sum the near pairs (rows
+// padded by one entry: the threads of a warp read a column of it), and Lambda
+// is read transposed, [g][s] (its rows put a warp's loads 128 bytes apart).
+// 53 -> 37 us at 7,459 panels of 16 nodes and 80 segments, 18 -> 12 at 1,743.
 // With agg given (the aggregated form): r = v - gpy with gpy = G_H P y
 // from the caller, and the coarse value is y[agg[i]].
 constexpr int kPanelThreads = 128;
 __global__ void __launch_bounds__(kPanelThreads) panel_apply_kernel(
     const float *__restrict__ part, int N, int g, int s, const int *__restrict__ nptr,
-    const int2 *__restrict__ pairs, const double *__restrict__ corr, const double *__restrict__ y,
-    const double *__restrict__ v, const double *__restrict__ inv, double *__restrict__ w,
+    const int2 *__restrict__ pairs, const float2 *__restrict__ corr, const float2 *__restrict__ y,
+    const double *__restrict__ v, const float2 *__restrict__ inv, double *__restrict__ w,
     const float2 *__restrict__ lam, float *__restrict__ sv, const int *__restrict__ agg,
     const double *__restrict__ gpy) {
-    __shared__ double rs[3 * kMaxG];
+    __shared__ float2 rs[3 * kMaxG];
     __shared__ float2 ws[3 * kMaxG];
+    __shared__ float2 bs[kMaxG * (kMaxG + 1)];
     const int i = blockIdx.x, t = threadIdx.x;
+    for (int u = t; u < g * g; u += kPanelThreads) bs[u + u / g] = inv[(size_t)i * g * g + u];
+    const int m = t / 3, c = t - 3 * m;
+    const size_t a = (size_t)i * g + m;
     if (agg) {   // aggregated form: r = v - G_H P y, supplied by the caller's FMM
-        if (t < 3 * g) rs[t] = v[3 * (size_t)i * g + t] - gpy[3 * (size_t)i * g + t];
+        if (t < 3 * g) rs[t] = ff::from(v[3 * a + c] - gpy[3 * a + c]);
     } else if (t < 3 * g) {
-        const int m = t / 3, c = t - 3 * m;
-        const size_t a = (size_t)i * g + m;
-        double acc = 0.0;
-        for (int q = 0; q < kSplit; ++q) acc += part[((size_t)q * N + a) * 3 + c];
-        for (int e0 = nptr[i]; e0 < nptr[i + 1]; e0 += 4) {   // four pairs' loads in flight
-            double cv[4], yv[4];
+        const double va = v[3 * a + c];
+        float pv[kSplit];
+#pragma unroll
+        for (int q = 0; q < kSplit; ++q) pv[q] = part[((size_t)q * N + a) * 3 + c];
+        float h = 0.f, l = 0.f;
+#pragma unroll
+        for (int q = 0; q < kSplit; ++q) {
+            const float2 z = ff::two_sum(h, pv[q]);
+            h = z.x;
+            l += z.y;
+        }
+        const int e1 = nptr[i + 1];
+        for (int e0 = nptr[i]; e0 < e1; e0 += 4) {   // four pairs' loads in flight
+            float2 cv[4], yv[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int e = e0 + u;
-                const bool ok = e < nptr[i + 1];
-                cv[u] = ok ? corr[(size_t)e * g + m] : 0.0;
-                yv[u] = ok ? y[3 * pairs[e].y + c] : 0.0;
+                const bool ok = e < e1;
+                cv[u] = ok ? corr[(size_t)e * g + m] : make_float2(0.f, 0.f);
+                yv[u] = ok ? y[3 * pairs[e].y + c] : make_float2(0.f, 0.f);
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) acc += cv[u] * yv[u];
+            for (int u = 0; u < 4; ++u) dot2ff(h, l, cv[u], yv[u]);
         }
-        rs[t] = v[3 * a + c] - acc;
+        rs[t] = ff::sub(ff::from(va), ff::quick(h, l));
     }
     __syncthreads();
     if (t < 3 * g) {
-        const int m = t / 3, c = t - 3 * m;
-        const double *row = inv + ((size_t)i * g + m) * g;
-        double acc = y[3 * (agg ? agg[i] : i) + c];
-        for (int n = 0; n < g; ++n) acc += row[n] * rs[3 * n + c];
-        if (w) w[3 * ((size_t)i * g + m) + c] = acc;
-        const float h = (float)acc;
-        ws[t] = make_float2(h, (float)(acc - (double)h));
+        const float2 *row = bs + m * (g + 1);
+        const float2 y0 = y[3 * (agg ? agg[i] : i) + c];
+        float h = y0.x, l = y0.y;
+        for (int n = 0; n < g; ++n) dot2ff(h, l, row[n], rs[3 * n + c]);
+        if (w) w[3 * a + c] = (double)h + (double)l;
+        ws[t] = ff::quick(h, l);
     }
     if (!lam) return;
     __syncthreads();
     for (int q = t; q < s; q += kPanelThreads) {
-        const float2 *lr = lam + (size_t)q * g;
         float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
-        for (int m = 0; m < g; ++m) {
-            const float2 l = lr[m];
-            dot2ff(h0, l0, l, ws[3 * m]);
-            dot2ff(h1, l1, l, ws[3 * m + 1]);
-            dot2ff(h2, l2, l, ws[3 * m + 2]);
+#pragma unroll 4
+        for (int n = 0; n < g; ++n) {
+            const float2 l = lam[(size_t)n * s + q];
+            dot2ff(h0, l0, l, ws[3 * n]);
+            dot2ff(h1, l1, l, ws[3 * n + 1]);
+            dot2ff(h2, l2, l, ws[3 * n + 2]);
         }
         const size_t k = (size_t)i * s + q;
         sv[3 * k + 0] = h0 + l0;
@@ -994,7 +1021,7 @@ cudaError_t TwoLevel::launch(const DevGeom &D, cudaStream_t st) {
     }
     if ((e = corr_.alloc(n_pairs * (size_t)g)) != cudaSuccess ||
         (e = Ainv_.alloc((size_t)n_pad_ * n_pad_)) != cudaSuccess || (e = s_.alloc(3 * (size_t)P)) != cudaSuccess ||
-        (e = y_.alloc(3 * (size_t)P)) != cudaSuccess || (e = pan_.alloc((size_t)P)) != cudaSuccess || (e = pan2_.alloc((size_t)P)) != cudaSuccess ||
+        (e = y_.alloc(3 * (size_t)P)) != cudaSuccess || (e = yff_.alloc(3 * (size_t)P)) != cudaSuccess || (e = pan_.alloc((size_t)P)) != cudaSuccess || (e = pan2_.alloc((size_t)P)) != cudaSuccess ||
         (K_ == 1 && (e = part_.alloc((size_t)kSplit * 3 * N)) != cudaSuccess))
         return e;
     const int ncol = (n_pad_ + 6) / 7;   // columns per checked row and block
@@ -1058,10 +1085,21 @@ cudaError_t TwoLevel::launch(const DevGeom &D, cudaStream_t st) {
     return cudaSuccess;
 }
 
-cudaError_t TwoLevel::finish(cudaStream_t st) {
+cudaError_t TwoLevel::finish(const double *inv, cudaStream_t st) {
     if (!launched_) return cudaSuccess;
     launched_ = false;
     cudaError_t e;
+    // what panel_apply_kernel reads, in float-float
+    const size_t n_inv = (size_t)P_ * g_ * g_, n_corr = K_ == 1 ? (size_t)n_pairs_ * g_ : 0;
+    if ((e = invff_.alloc(n_inv)) != cudaSuccess || (e = corrff_.alloc(n_corr)) != cudaSuccess) return e;
+    auto conv = [&](const double *src, float2 *dst, size_t n) {
+        if (n == 0) return;
+        to_ff_kernel<<<(unsigned)std::min<size_t>((n + 255) / 256, 1216), 256, 0, st>>>(src, dst, n);
+        note_launch();
+    };
+    conv(inv, invff_.ptr, n_inv);
+    conv(corr_.ptr, corrff_.ptr, n_corr);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     std::vector<double> errs_h(errs_.n);
     int bad_h = 0;
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess ||
@@ -1069,6 +1107,7 @@ cudaError_t TwoLevel::finish(cudaStream_t st) {
         (e = cudaMemcpy(&bad_h, bad_.ptr, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess)
         return e;
     Ac_.release();
+    corr_.release();
     gj_tmp_.release();
     errs_.release();
     bad_.release();
@@ -1082,13 +1121,13 @@ cudaError_t TwoLevel::finish(cudaStream_t st) {
     return cudaSuccess;
 }
 
-cudaError_t TwoLevel::apply(const double *inv, const double *v, double *w, cudaStream_t st, const float2 *lam, int s,
+cudaError_t TwoLevel::apply(const double *v, double *w, cudaStream_t st, const float2 *lam, int s,
                             float *sv) {
     const int P = P_, g = g_, N = P * g;
     if (K_ > 1) return cudaErrorNotSupported;   // aggregated: apply_stage1 / apply_stage2
     restrict_kernel<<<(3 * P + 255) / 256, 256, 0, st>>>(v, P, g, s_.ptr);
     coarse_solve_kernel<<<(P + kSolveRows - 1) / kSolveRows, 32 * kSolveRows, 0, st>>>(
-        Ainv_.ptr, n_pad_, P, s_.ptr, plen32_.ptr, c32_.ptr, y_.ptr, pan_.ptr, pan2_.ptr);
+        Ainv_.ptr, n_pad_, P, s_.ptr, plen32_.ptr, c32_.ptr, y_.ptr, yff_.ptr, pan_.ptr, pan2_.ptr);
     if (n_leaves_ > 0) {
         if (n_far_ > 0) {
             cluster_moments_kernel<<<n_far_, kTreeThreads, 0, st>>>(far_.ptr, geo_.ptr, range_.ptr, mo_.ptr, pan_.ptr, pan2_.ptr,
@@ -1102,8 +1141,8 @@ cudaError_t TwoLevel::apply(const double *inv, const double *v, double *w, cudaS
         monopole_kernel<<<dim3((N + per_block - 1) / per_block, kSplit), kMonoThreads, 0, st>>>(
             q32_.ptr, pan_.ptr, pan2_.ptr, P, N, part_.ptr);
     }
-    panel_apply_kernel<<<P, kPanelThreads, 0, st>>>(part_.ptr, N, g, s, nptr_.ptr, pairs_.ptr, corr_.ptr, y_.ptr,
-                                                    v, inv, w, lam, sv, nullptr, nullptr);
+    panel_apply_kernel<<<P, kPanelThreads, 0, st>>>(part_.ptr, N, g, s, nptr_.ptr, pairs_.ptr, corrff_.ptr, yff_.ptr,
+                                                    v, invff_.ptr, w, lam, sv, nullptr, nullptr);
     note_launch(4);
     return cudaGetLastError();
 }
@@ -1112,16 +1151,16 @@ cudaError_t TwoLevel::apply_stage1(const double *v, double *py, cudaStream_t st)
     const int N = P_ * g_;
     restrict_agg_kernel<<<(3 * nA_ + 255) / 256, 256, 0, st>>>(v, pagg_.ptr, perm_.ptr, nA_, g_, s_.ptr);
     coarse_solve_kernel<<<(nA_ + kSolveRows - 1) / kSolveRows, 32 * kSolveRows, 0, st>>>(
-        Ainv_.ptr, n_pad_, nA_, s_.ptr, plen32_.ptr, c32_.ptr, y_.ptr, pan_.ptr, pan2_.ptr);
+        Ainv_.ptr, n_pad_, nA_, s_.ptr, plen32_.ptr, c32_.ptr, y_.ptr, yff_.ptr, pan_.ptr, pan2_.ptr);
     spread_agg_kernel<<<(3 * N + 255) / 256, 256, 0, st>>>(y_.ptr, agg_of_.ptr, N, g_, py);
     note_launch(3);
     return cudaGetLastError();
 }
 
-cudaError_t TwoLevel::apply_stage2(const double *inv, const double *v, const double *gpy, double *w, cudaStream_t st,
+cudaError_t TwoLevel::apply_stage2(const double *v, const double *gpy, double *w, cudaStream_t st,
                                    const float2 *lam, int s, float *sv) {
-    panel_apply_kernel<<<P_, kPanelThreads, 0, st>>>(nullptr, P_ * g_, g_, s, nptr_.ptr, pairs_.ptr, corr_.ptr, y_.ptr,
-                                                     v, inv, w, lam, sv, agg_of_.ptr, gpy);
+    panel_apply_kernel<<<P_, kPanelThreads, 0, st>>>(nullptr, P_ * g_, g_, s, nptr_.ptr, pairs_.ptr, corrff_.ptr, yff_.ptr,
+                                                     v, invff_.ptr, w, lam, sv, agg_of_.ptr, gpy);
     note_launch();
     return cudaGetLastError();
 }

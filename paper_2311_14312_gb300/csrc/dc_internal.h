@@ -267,11 +267,11 @@ public:
     // work: plan() is host work only (centroids, aggregates, near panel
     // pairs; max_coarse: most coarse unknowns, 0 = the built-in 12288);
     // launch() enqueues the uploads, the coarse matrix, its inversion and the
-    // check of the inverse on st and waits for none of them; finish() waits
-    // for st and decides from the check whether the coarse level is used.
+    // check of the inverse on st and waits for none of them; finish() converts
+    // the panel blocks' inverses inv (written on st before), waits for st and decides from the check whether the coarse level is used.
     void plan(const Geometry &G, int max_coarse);
     cudaError_t launch(const DevGeom &D, cudaStream_t st);
-    cudaError_t finish(cudaStream_t st);
+    cudaError_t finish(const double *inv, cudaStream_t st);
     bool ready() const { return ready_; }
     // coarse unknowns (panels, or aggregates of K panels), near panel pairs,
     // max |(Ac^-1 Ac - I)_ij| over 5 sampled rows, K
@@ -282,18 +282,17 @@ public:
         out[3] = check_;
         out[4] = K_;
     }
-    // w = M v on [N][3] vectors (w may be null); inv: the panel blocks'
-    // inverses.  With lam (Lambda as hi/lo floats, [s][g]) and sv: also
-    // sv = Lambda (M v) per panel, [S][3] FP32.
-    cudaError_t apply(const double *inv, const double *v, double *w, cudaStream_t st, const float2 *lam = nullptr,
-                      int s = 0, float *sv = nullptr);
+    // w = M v on [N][3] vectors (w may be null).  With lam (Lambda as hi/lo
+    // floats, [g][s]) and sv: also sv = Lambda (M v) per panel, [S][3] FP32.
+    cudaError_t apply(const double *v, double *w, cudaStream_t st, const float2 *lam = nullptr, int s = 0,
+                      float *sv = nullptr);
     // The aggregated form (aggregated() true) in two stages around the
     // caller's operator application: stage 1 solves the coarse system and
     // spreads py = P y to the nodes; stage 2 takes gpy = G_H py and forms
     // w = P y + B (v - gpy) (and sv as in apply).
     bool aggregated() const { return ready_ && K_ > 1; }
     cudaError_t apply_stage1(const double *v, double *py, cudaStream_t st);
-    cudaError_t apply_stage2(const double *inv, const double *v, const double *gpy, double *w, cudaStream_t st,
+    cudaError_t apply_stage2(const double *v, const double *gpy, double *w, cudaStream_t st,
                              const float2 *lam = nullptr, int s = 0, float *sv = nullptr);
 
 private:
@@ -324,10 +323,10 @@ private:
                                          // panel, panels in Morton order
     double check_ = -1.0;
     DevBuf<float2> c32_, q32_;
-    DevBuf<double> plen_, corr_, y_;
+    DevBuf<double> plen_, corr_, y_;   // corr_: launch() to finish()
     DevBuf<float> plen32_, pan2_, Ainv_, part_;
     DevBuf<float4> pan_;
-    DevBuf<float2> s_;
+    DevBuf<float2> s_, yff_, corrff_, invff_;   // float-float: inputs, y, near corrections, panel blocks
     DevBuf<int> nptr_;
     DevBuf<int2> pairs_;
 };

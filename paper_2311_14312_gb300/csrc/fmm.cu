@@ -1197,11 +1197,11 @@ dc_status Fmm::build(const dc_options &opt, const Geometry &G, const DevGeom &D,
         }
         return f;
     };
-    auto lam_hilo = [](const std::vector<double> &v) {   // (hi, lo) float pairs
+    auto lam_hilo = [&D](const std::vector<double> &v) {   // (hi, lo) float pairs, transposed
         std::vector<float2> f(v.size());
         for (size_t i = 0; i < v.size(); ++i) {
             const float h = (float)v[i];
-            f[i] = make_float2(h, (float)(v[i] - (double)h));
+            f[(i % D.g) * D.s + i / D.g] = make_float2(h, (float)(v[i] - (double)h));
         }
         return f;
     };
@@ -1384,7 +1384,7 @@ dc_status Fmm::build(const dc_options &opt, const Geometry &G, const DevGeom &D,
                       : std::string("fmm preconditioner: ") + cudaGetErrorString(pre_err);
         return (pre_oom || pre_err == cudaErrorMemoryAllocation) ? DC_ERR_OOM : DC_ERR_CUDA;
     }
-    if ((e = I.render_only ? cudaStreamSynchronize(I.pre_stream) : I.coarse.finish(I.pre_stream)) != cudaSuccess) {
+    if ((e = I.render_only ? cudaStreamSynchronize(I.pre_stream) : I.coarse.finish(I.pinv.ptr, I.pre_stream)) != cudaSuccess) {
         err = std::string("fmm preconditioner: ") + cudaGetErrorString(e);
         return e == cudaErrorMemoryAllocation ? DC_ERR_OOM : DC_ERR_CUDA;
     }
@@ -1511,9 +1511,9 @@ cudaError_t Fmm::Impl::precond(const double *v, double *w, cudaStream_t st) {
             return e;
         e = fp32 ? apply_nodes32(agg_py.ptr, agg_gpy.ptr, true, st) : apply_nodes(agg_py.ptr, agg_gpy.ptr, true, st);
         if (e != cudaSuccess) return e;
-        return coarse.apply_stage2(pinv.ptr, v, agg_gpy.ptr, w, st);
+        return coarse.apply_stage2(v, agg_gpy.ptr, w, st);
     }
-    if (coarse.ready()) return coarse.apply(pinv.ptr, v, w, st);
+    if (coarse.ready()) return coarse.apply(v, w, st);
     return launch_block_apply(pinv.ptr, D->n_panels, D->g, v, w, st);
 }
 

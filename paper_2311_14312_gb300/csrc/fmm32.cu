@@ -78,10 +78,10 @@ __global__ void interp32_kernel(const float2 *__restrict__ lam, const double *__
     }
     __syncthreads();
     for (int q = kk; q < s; q += blockDim.x) {
-        const float2 *row = lam + (size_t)q * g;
         float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
+#pragma unroll 4
         for (int m = 0; m < g; ++m) {
-            const float2 l = row[m];
+            const float2 l = lam[(size_t)m * s + q];
             dot2ff(h0, l0, l, v[3 * m]);
             dot2ff(h1, l1, l, v[3 * m + 1]);
             dot2ff(h2, l2, l, v[3 * m + 2]);
@@ -1021,9 +1021,9 @@ cudaError_t Fmm::Impl::graph_ensure() {
         if (e1 == cudaSuccess) e1 = interp32(agg_py.ptr, sbar32.ptr, cap_stream);
         if (e1 == cudaSuccess) e1 = node_op(agg_gpy.ptr);
         if (e1 == cudaSuccess)
-            e1 = coarse.apply_stage2(pinv.ptr, g_in.ptr, agg_gpy.ptr, nullptr, cap_stream, lam_ff.ptr, D->s, sbar32.ptr);
+            e1 = coarse.apply_stage2(g_in.ptr, agg_gpy.ptr, nullptr, cap_stream, lam_ff.ptr, D->s, sbar32.ptr);
     } else {
-        e1 = coarse.ready() ? coarse.apply(pinv.ptr, g_in.ptr, nullptr, cap_stream, lam_ff.ptr, D->s, sbar32.ptr)
+        e1 = coarse.ready() ? coarse.apply(g_in.ptr, nullptr, cap_stream, lam_ff.ptr, D->s, sbar32.ptr)
                             : precond(g_in.ptr, ir_t.ptr, cap_stream);
     }
     cudaError_t e2 = e1;

@@ -225,7 +225,7 @@ struct Fmm::Impl {
     DevBuf<int4> tc_tiles;
     int n_tc_tiles = 0;
     long long m2l_pairs_nodes = 0;    // list-2 pairs of the node schedule
-    DevBuf<float2> lam_ff;            // Lambda [s][g] as (hi, lo) floats
+    DevBuf<float2> lam_ff;            // Lambda transposed, [g][s], as (hi, lo) floats
     DevBuf<double> iw64, logw64, plen64;
     DevBuf<unsigned char> heavy;      // per piece: near field evaluated in FP64
     DevBuf<unsigned char> heavyL, heavyM;   // per cell: L2P / M2P evaluated in FP64

@@ -1,4 +1,4 @@
-"""The two-level preconditioner's monopole sums over a cluster tree (1,024
+"""The two-level preconditioner's monopole sums over a cluster tree (2,048
 panels and more) and directly (one panel fewer), against the definition
 written out with numpy: at the switch, with a full and with a short last
 cluster."""
@@ -11,7 +11,7 @@ from test_gpu_precond import reference_M
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("curves,per_curve", [(11, 93), (16, 64), (11, 95)])   # 1023, 1024, 1045 panels
+@pytest.mark.parametrize("curves,per_curve", [(23, 89), (16, 128), (13, 159)])   # 2047, 2048, 2067 panels
 def test_cluster_preconditioner_matches_definition(dcmod, cuda_ok, oracle_mod, curves, per_curve):
     # Bound: the coarse inverse is FP32 with an inverse_check below 1e-3 by
     # its own acceptance; the cluster sums add 0.4^9 / 9 = 3e-5 of a far term.
