@@ -239,7 +239,11 @@ __global__ void __launch_bounds__(kChunk) p2m_kernel(TreeView<T> t, PS ps, const
 // m2m_reduce_kernel adds up in chunk order.  For P1 <= 16 the half-warps
 // take alternate pairs (lane k + 16 h holds coefficient k of pair 2 i + h)
 // and are added at the end; above 16 lane k holds coefficient k of every
-// pair.  The binomial table is staged in shared memory.
+// pair.  The binomial table is staged in shared memory, its rows padded: at
+// 32 entries a row all lanes read one bank, 13 passes for every term.
+// With that and the next pair's loads ahead of this one's sum: 80 -> 59 us for
+// 119,344 nodes (order 12, cold), 25 -> 18 for 27,888; the inner operator with
+// the preconditioner 700 -> 659 and 181 -> 167.
 constexpr int kMultiLeaves = 16;
 constexpr int kMultiWarps = 4;
 
@@ -251,11 +255,11 @@ __global__ void __launch_bounds__(32 * kMultiWarps) m2m_multi_kernel(const float
                                                                      typename V2<T>::type *__restrict__ M,
                                                                      typename V2<T>::type *__restrict__ partial) {
     using C = typename V2<T>::type;
+    constexpr int kRow = 33;   // odd: the lanes of a warp read a column
     __shared__ C zp[kMultiWarps][32];
-    __shared__ T rp[kMultiWarps][32];
     __shared__ C ms[kMultiWarps][2][96];
-    __shared__ T sbin[32 * 32];
-    for (int i = threadIdx.x; i < P1 * 32; i += blockDim.x) sbin[i] = binom[i];
+    __shared__ T sbin[32 * kRow];
+    for (int i = threadIdx.x; i < P1 * 32; i += blockDim.x) sbin[i + i / 32] = binom[i];
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ci = blockIdx.x * kMultiWarps + warp;
@@ -267,18 +271,26 @@ __global__ void __launch_bounds__(32 * kMultiWarps) m2m_multi_kernel(const float
     const int h = halves == 2 ? lane >> 4 : 0, k = lane - h * span;
     C acc[3];
     for (int c = 0; c < 3; ++c) acc[c] = mk<T>(0, 0);
-    const int nM = 3 * P1;
-    for (int e0 = ch.y; e0 < ch.y + ch.z; e0 += halves) {
-        const int e = e0 + h;
-        const bool has = e < ch.y + ch.z;
+    const int nM = 3 * P1, end = ch.y + ch.z;
+    // the next pair's shift and moments are fetched while this one is summed
+    float4 geo = make_float4(0.f, 0.f, 0.f, 0.f);
+    C mk0 = mk<T>(0, 0), mk1 = mk0, mk2 = mk0;
+    auto fetch = [&](int e) {
+        if (e >= end || k >= P1) return;
+        geo = pair_geo[e];
+        const C *src = M + (size_t)pair_leaf[e] * nM + k;
+        mk0 = src[0];
+        mk1 = src[P1];
+        mk2 = src[2 * P1];
+    };
+    fetch(ch.y + h);
+    for (int e0 = ch.y; e0 < end; e0 += halves) {
+        const bool on = e0 + h < end && k < P1;
         // d^k and rho^k by binary powering (the pair's shift d and scale rho
         // were formed once per drawing)
-        const float4 geo = has ? pair_geo[e] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const C d = mk<T>((T)geo.x, (T)geo.y);
-        const T rho = (T)geo.z;
-        C pz = mk<T>(1, 0), bz = d;
-        T pr = 1, br = rho;
-        for (int bit = 1; bit < 32; bit <<= 1) {
+        C pz = mk<T>(1, 0), bz = mk<T>((T)geo.x, (T)geo.y);
+        T pr = 1, br = (T)geo.z;
+        for (int bit = 1; bit < span; bit <<= 1) {
             if (k & bit) {
                 pz = cmul(pz, bz);
                 pr *= br;
@@ -287,20 +299,20 @@ __global__ void __launch_bounds__(32 * kMultiWarps) m2m_multi_kernel(const float
             br *= br;
         }
         __syncwarp();
+        C *m = ms[warp][h];
         zp[warp][lane] = pz;                         // [h][k] = lane
-        rp[warp][lane] = pr;
-        if (has) {
-            const C *src = M + (size_t)pair_leaf[e] * nM;
-            for (int i = k; i < nM; i += span) ms[warp][h][i] = src[i];
+        if (on) {
+            m[k] = cscl(mk0, pr);
+            m[P1 + k] = cscl(mk1, pr);
+            m[2 * P1 + k] = cscl(mk2, pr);
         }
+        fetch(e0 + halves + h);
         __syncwarp();
-        if (has && k < P1) {
-            const T *bk = sbin + k * 32;
+        if (on) {
+            const T *bk = sbin + k * kRow;
             const C *z = zp[warp] + h * span;
-            const T *r = rp[warp] + h * span;
-            const C *m = ms[warp][h];
             for (int j = 0; j <= k; ++j) {
-                const C co = cscl(z[k - j], bk[j] * r[j]);
+                const C co = cscl(z[k - j], bk[j]);
                 for (int c = 0; c < 3; ++c) cfma(acc[c], co, m[c * P1 + j]);
             }
         }
