@@ -148,12 +148,13 @@ __device__ __forceinline__ float2 atan2(const Tables &T, float2 y, float2 x) {
 
 // ilog = int log|p - q| dS and phi = the subtended angle of the segment from
 // a to b (relative to the target), half length vector not needed: d = b - a
-// and len = |d| are the piece's own.
+// and len = |d| are the piece's own.  own: the target is a node of the piece's
+// segment, phi = 0.
 __device__ __forceinline__ void pair(const Tables &T, float2 ax, float2 ay, float2 bx, float2 by, float2 dx, float2 dy,
-                                     float2 len, float2 &ilog, float2 &phi) {
+                                     float2 len, float2 &ilog, float2 &phi, bool own = false) {
     const float2 mx = scale(add(ax, bx), 0.5f), my = scale(add(ay, by), 0.5f);   // midpoint
     const float2 r2 = dot(mx, mx, my, my);
-    if (16.f * len.x * len.x < r2.x) {
+    if (!own && 16.f * len.x * len.x < r2.x) {
         // series in zeta = eta^2, eta = d / (2 m), |zeta| < 1/64:
         //   ilog = len (log|m| - Re sum_k zeta^k / (2k (2k+1))),  phi = 2 Im eta sum_k zeta^k / (2k+1)
         // the first two terms in float-float, the rest (below 10^-7) in FP32
@@ -192,7 +193,7 @@ __device__ __forceinline__ void pair(const Tables &T, float2 ax, float2 ay, floa
         return;
     }
     const float2 cr = dot(ax, by, neg(ay), bx), dt = dot(ax, bx, ay, by);
-    phi = (cr.x == 0.f && dt.x == 0.f) ? make_float2(0.f, 0.f) : atan2(T, cr, dt);   // at an end point: 0
+    phi = own || (cr.x == 0.f && dt.x == 0.f) ? make_float2(0.f, 0.f) : atan2(T, cr, dt);   // own, or at an end point: 0
     const float2 ra2 = dot(ax, ax, ay, ay), rb2 = dot(bx, bx, by, by), il = inv(len);
     const float2 s1 = mul(dot(ax, dx, ay, dy), il), s2 = mul(dot(bx, dx, by, dy), il);
     float2 la = make_float2(0.f, 0.f), lb = la;

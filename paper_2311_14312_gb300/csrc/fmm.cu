@@ -563,25 +563,45 @@ cudaError_t Fmm::Impl::build_near(cudaStream_t st) {
     cudaError_t e = cudaMemGetInfo(&fr, &tot);
     if (e != cudaSuccess) return e;
     if (need > fr / 4) return cudaSuccess;
-    if ((e = near_g64.alloc((size_t)near_total)) != cudaSuccess) return e;
-    if ((e = near_f64.alloc((size_t)near_total)) != cudaSuccess) return e;
+    if (fp32 && (e = near_g32.alloc((size_t)near_total)) != cudaSuccess) return e;
+    // The FP64 node operator reads near and far coefficients in float-float
+    // when both are stored; the near ones are then formed so at once.  Not with
+    // large leaves (near_coef_ff_kernel says why), nor on a canvas so small
+    // that the square of a coordinate's last bit leaves the floats' range, or
+    // so large that a squared distance might: FP64, narrowed.
+    const size_t need_far = (size_t)far_blocks * (P1 * sizeof(double2) + (fp32 ? P1i * sizeof(float2) : 0));
+    const bool want_far = far_blocks > 0 && need_far <= (fr - need) / 4;
+    const bool ff_direct =
+        want_far && opt.leaf_size <= evalnodes::kFfLeaf && tree.w0 >= 0x1p-7 && tree.w0 <= 0x1p20;
     evalnodes::NodeArgs<double> a = node_args64(nt_items4.ptr, nt_xy.ptr, nt_own1.ptr, nt_own2.ptr,
                                                 nt_perm.ptr, nullptr, nullptr, 0, 0, nullptr);
-    evalnodes::near_coef_kernel<<<n_nt_items4, 32 * evalnodes::kWarps, 0, st>>>(a, near_off.ptr,
-                                                                               near_g64.ptr, near_f64.ptr);
-    note_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (fp32) {
-        if ((e = near_g32.alloc((size_t)near_total)) != cudaSuccess) return e;
-        narrow_real_kernel<<<4 * n_sms, 256, 0, st>>>(near_g64.ptr, near_g32.ptr, near_total);
+    if (want_far && ((e = near_gff.alloc((size_t)near_total)) != cudaSuccess ||
+                     (e = near_fff.alloc((size_t)near_total)) != cudaSuccess))
+        return e;
+    if (ff_direct) {
+        evalnodes::near_coef_ff_kernel<<<std::min(n_nt_items4, 6 * n_sms), 32 * evalnodes::kWarps, 0, st>>>(
+            a, near_off.ptr, n_nt_items4, near_gff.ptr, near_fff.ptr, fp32 ? near_g32.ptr : nullptr);
         note_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    } else {
+        if ((e = near_g64.alloc((size_t)near_total)) != cudaSuccess) return e;
+        if ((e = near_f64.alloc((size_t)near_total)) != cudaSuccess) return e;
+        evalnodes::near_coef_kernel<<<n_nt_items4, 32 * evalnodes::kWarps, 0, st>>>(a, near_off.ptr,
+                                                                                   near_g64.ptr, near_f64.ptr);
+        note_launch();
+        if (fp32) {
+            narrow_real_kernel<<<4 * n_sms, 256, 0, st>>>(near_g64.ptr, near_g32.ptr, near_total);
+            note_launch();
+        }
+        if (want_far) {
+            d2ff_kernel<<<4 * n_sms, 256, 0, st>>>(near_g64.ptr, near_gff.ptr, near_total);
+            d2ff_kernel<<<4 * n_sms, 256, 0, st>>>(near_f64.ptr, near_fff.ptr, near_total);
+            note_launch(2);
+        }
     }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     near_ready = true;
     // far-field coefficients (L2P and list-3 M2P at the nodes), when they fit too
-    const size_t need_far = (size_t)far_blocks * (P1 * sizeof(double2) + (fp32 ? P1i * sizeof(float2) : 0));
-    if ((e = cudaMemGetInfo(&fr, &tot)) != cudaSuccess) return e;
-    if (far_blocks <= 0 || need_far > fr / 4) return cudaSuccess;
+    if (!want_far) return cudaSuccess;
     if ((e = far64.alloc((size_t)far_blocks * P1)) != cudaSuccess) return e;
     far_coef_launch(st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -592,15 +612,9 @@ cudaError_t Fmm::Impl::build_near(cudaStream_t st) {
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     far_ready = true;
-    // the FP64 node operator reads both in float-float (same sizes)
-    if ((e = near_gff.alloc((size_t)near_total)) != cudaSuccess ||
-        (e = near_fff.alloc((size_t)near_total)) != cudaSuccess ||
-        (e = farff.alloc((size_t)far_blocks * P1)) != cudaSuccess)
-        return e;
-    d2ff_kernel<<<4 * n_sms, 256, 0, st>>>(near_g64.ptr, near_gff.ptr, near_total);
-    d2ff_kernel<<<4 * n_sms, 256, 0, st>>>(near_f64.ptr, near_fff.ptr, near_total);
+    if ((e = farff.alloc((size_t)far_blocks * P1)) != cudaSuccess) return e;
     passes::rows_to_ff_kernel<<<4 * n_sms, 256, 0, st>>>(far64.ptr, farff.ptr, (size_t)far_blocks * P1);
-    note_launch(3);
+    note_launch();
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
     near_g64.release();
     near_f64.release();
