@@ -156,8 +156,8 @@ class ClockSampler:
 def traffic_for_eval_kernel():
     """DRAM bytes per launch of the eval kernel from a committed ncu
     summary, valid only while the kernel source is unchanged."""
-    src = os.path.join(ROOT, "paper_2311_14312_gb300", "csrc", "fmm32.cu")
-    path = os.path.join(ROOT, "profiles", "eval32_traffic.json")
+    src = os.path.join(ROOT, "paper_2311_14312_gb300", "csrc", "rendertiles.cuh")
+    path = os.path.join(ROOT, "profiles", "render32_traffic.json")
     try:
         ref = json.load(open(path))
         sha = hashlib.sha1(open(src, "rb").read()).hexdigest()
@@ -488,7 +488,7 @@ def run_ours(args):
             "render_mpix_s": npx / (statistics.mean(render_ms) * 1e-3) / 1e6,
             "gmres_iters": list(st.iters), "gmres_rel_resid": max(st.rel_resid),
             "plain_form": plain,
-            "roofline": {"bound": "alu", "kernel": "eval32_kernel<0> (L2P + M2P + P2P per pixel)",
+            "roofline": {"bound": "alu", "kernel": "render32_kernel (flops of the direct L2P + M2P + P2P per pixel)",
                          "achieved": achieved, "peak": fp32["tflops"], "unit": "TFLOP/s",
                          "frac": (achieved / fp32["tflops"]) if achieved else None,
                          "peak_source": f"measured: FP32 FMA chains on this GPU ({props.multi_processor_count} "
@@ -601,7 +601,7 @@ def run_large(args):
             "build_s": build_s, "solve_ms": statistics.mean(solve_ms), "render_ms": statistics.mean(render_ms),
             "render_mpix_s": npx / (statistics.mean(render_ms) * 1e-3) / 1e6, "gmres_iters": list(st.iters),
             "gmres_rel_resid": max(st.rel_resid), "plain_form": plain,
-            "roofline": {"bound": "alu", "kernel": "eval32_kernel<0> (L2P + M2P + P2P per pixel)",
+            "roofline": {"bound": "alu", "kernel": "render32_kernel (flops of the direct L2P + M2P + P2P per pixel)",
                          "achieved": achieved, "peak": fp32["tflops"], "unit": "TFLOP/s",
                          "frac": (achieved / fp32["tflops"]) if achieved else None, "traffic": None,
                          "eval_ms": rs.ms_eval, "p2p_pairs": rs.p2p_pairs, "m2p_pairs": rs.m2p_pairs},

@@ -127,10 +127,10 @@ typedef struct {
                               (0 = 2) ...                                    */
     double adapt_max_len;  /* ... and no panel longer than this (0 = 0.5);
                               measured on 256-point polylines per curve      */
-    int eval_tile;         /* DC_FORM_FMM32: pixel tile of one block of the
-                              render's evaluation kernel: 0 = 8 x 8 (default),
-                              1 = 16 x 8, 2 = 16 x 16, 3 = 32 x 8 (width x
-                              height)                                         */
+    int eval_tile;         /* DC_FORM_FMM32: largest pixel rectangle of one
+                              block of the render's evaluation kernel: 0 =
+                              sized by the leaf (default), 1 = 16 x 8, 2 =
+                              16 x 16, 3 = 32 x 8 (width x height)            */
     int aa_levels;         /* quadtree anti-aliasing of the render (Sec. 7):
                               0 = off (centre samples, default); m in [1, 6]:
                               a pixel whose closed square meets a segment is
@@ -191,9 +191,11 @@ typedef struct {
     long long p2p_pairs;   /* (pixel, clipped piece) pairs of list 1         */
     long long m2p_pairs;   /* (pixel, cell) pairs of list 3                  */
     long long m2l_pairs;   /* cell pairs of list 2 in the passes             */
-    double eval_flops;     /* algorithmic flops of the evaluation kernels:
-                              45 per near-field pair, 24 (p + 1) per L2P and
-                              per list-3 M2P (3 colour channels)              */
+    double eval_flops;     /* algorithmic flops of the direct evaluation: 45
+                              per near-field pair, 24 (p + 1) per L2P and per
+                              list-3 M2P (3 colour channels); the FP32 kernel
+                              samples what is far from a rectangle and does
+                              fewer                                           */
     long long aa_pixels;   /* pixels refined by the anti-aliasing (aa_levels) */
     long long aa_samples;  /* their samples                                  */
     double ms_aa;          /* device time of the anti-aliasing pass          */
@@ -318,7 +320,7 @@ dc_status dc_eval_points_noalloc(dc_ctx *ctx, int n, const double *xy_dev, doubl
 /* ---------------------------------------------------------------------
  * Autotuning of the chosen form (no counterpart in the paper, which gives
  * neither the leaf size b nor K): candidates are the cross product of leaf
- * sizes x inner orders p_inner x pixel tile shapes (eval_tile); each is
+ * sizes x inner orders p_inner x pixel rectangles (eval_tile); each is
  * built on the context's drawing, warmed up, and timed (solve + render of
  * the viewports, CUDA events on the context's stream, best of `repeats`);
  * its FP32 pixels are compared with a plain FP64 FMM render of the same
