@@ -229,6 +229,7 @@ struct EvalArgs32 {
     // persistent launch: the item counter (zero at launch) and the item count
     int *queue;
     int n_items;
+    float side;            // distance from a piece below which its side is decided in FP64
     // list mode
     const float2 *q32;
     const double *q64;
@@ -1066,6 +1067,8 @@ cudaError_t Fmm::Impl::render_tiles32(int n_tiles, void *rgb, int rgb_dtype,
     a.t = dt32();
     a.t64 = dt();
     a.rects = tiles.ptr;
+    a.side = (float)(rtiles::kSideBound * std::max({std::fabs(tree.x0), std::fabs(tree.y0), std::fabs(tree.x0 + tree.w0),
+                                                    std::fabs(tree.y0 + tree.w0)}));
     a.P1 = P1;
     a.M = M32.ptr;
     a.L = L32.ptr;

@@ -39,8 +39,9 @@ constexpr float kSep = 2.5f;       // far: at least this many radii from the cen
 // is 0.2^16 / 16 = 4e-13
 constexpr float kSepBig = 5.f;
 constexpr float kMaxRadius = 0.36f, kMaxRadiusBig = 0.18f;   // R in leaf widths (local expansion)
-// distance from a piece (world units; coordinates are of order one) below which
-// its side is decided in FP64: the (hi, lo) pairs hold 48 bits
+// distance from a piece, times the largest coordinate of the canvas, below which
+// its side is decided in FP64: the (hi, lo) pairs hold 48 bits (3.6e-15 of the
+// coordinate; 17 times that covers the differences and products of cross_ff)
 constexpr float kSideBound = 6e-14f;
 constexpr int kMinSampled = 48;    // rectangles of fewer pixels are evaluated directly
 constexpr int kStaged = 64;        // near pieces staged per warp
@@ -689,7 +690,7 @@ __device__ __forceinline__ void item(const EvalArgs32 &a, int it, BlockMem &B) {
                                 bool exact = false;
                                 if (pair_beside(ax, ay, bx, by, C.x, cr)) {
                                     cr = cross_ff(A, Bl, xh, xl, yh, yl);
-                                    exact = fabsf(cr) < kSideBound * F.iw * C.x;
+                                    exact = fabsf(cr) < a.side * F.iw * C.x;
                                 }
                                 if (exact) {   // closer than the (hi, lo) coordinates resolve
                                     w = pair64(a.t64.pc + 4 * (size_t)__float_as_int(D.w), vp.x0 + (c + 0.5) * vp.dx,

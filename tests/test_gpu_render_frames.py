@@ -1,0 +1,70 @@
+"""The FP32 form's pixel rectangles where their frames are strained: canvases
+far from the origin and in pixel units, where a pixel's side of a curve is
+finer than the (hi, lo) coordinates.  Tolerance: the form's 1e-5 of the
+field."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from dc_synth import drawing_by_name, random_node_values
+
+pytestmark = pytest.mark.gpu
+
+DOMAIN = (-0.5, -0.5, 1.5, 1.5)
+
+
+def _render(dcmod, ctx, views):
+    import torch
+    out = torch.empty((sum(v[4] * v[5] for v in views), 3), dtype=torch.float64, device="cuda")
+    ctx.render_viewport(views, out)
+    torch.cuda.synchronize()
+    return out.cpu().numpy()
+
+
+def library_discretisation(dcmod, O, d):
+    """The oracle's discretisation with the library's own end points, which
+    differ from it by some 1e-13."""
+    disc = O.discretise(d)
+    own = dcmod.aux_discretise(d.ctrl, d.panel_ptr, d.panel_start, d.colours, d.g, d.s_per_panel)
+    return dataclasses.replace(disc, node_xy=own["node_xy"], seg_xy=own["seg_xy"], seg_w=own["seg_w"])
+
+
+def line_distance(seg, pts):
+    """Distances of pts from the nearest of the segments, in extended precision."""
+    q = np.asarray(pts, np.longdouble)[:, None]
+    a, b = np.asarray(seg[:, :2], np.longdouble)[None], np.asarray(seg[:, 2:], np.longdouble)[None]
+    ab = b - a
+    t = np.clip(((q - a) * ab).sum(2) / (ab * ab).sum(2), 0, 1)
+    e = a + t[..., None] * ab - q
+    return np.sqrt((e * e).sum(2)).min(1).astype(float)
+
+
+@pytest.mark.parametrize("scale,shift", [(1.0, 0.0), (2048.0, 0.0), (2.0 ** 16, 0.0), (1.0, 300.0), (64.0, -5000.0)])
+def test_side_of_a_curve_far_from_the_origin(dcmod, cuda_ok, oracle_mod, scale, shift):
+    O = oracle_mod
+    d = drawing_by_name("mixed16")
+    d = dataclasses.replace(d, ctrl=d.ctrl * scale + shift)
+    disc = library_discretisation(dcmod, O, d)
+    up, um = O.boundary_values(d, disc)
+    sig = random_node_values(disc.n_nodes, seed=35, scale=1.0 / scale)
+    ctx = dcmod.Context(form="fmm32", g=d.g, s_per_panel=d.s_per_panel, p=24,
+                        domain=tuple(shift + scale * c for c in DOMAIN))
+    ctx.build_drawing(d)
+    ctx.set_density(sig)
+    big = np.abs(disc.seg_xy).max()
+    ulp = 2.0 ** (np.floor(np.log2(big)) - 52)
+    views = []
+    for k in range(5, disc.n_segments, 211):
+        x1, y1, x2, y2 = disc.seg_xy[k]
+        mx, my = np.round(0.5 * (x1 + x2) / ulp) * ulp, np.round(0.5 * (y1 + y2) / ulp) * ulp
+        for w, h, px in ((16, 16, 2 * ulp), (16, 16, 16 * ulp), (7, 6, 8 * ulp)):   # sampled and direct
+            views.append((mx - w // 2 * px, my - h // 2 * px, mx + (w - w // 2) * px, my + (h - h // 2) * px, w, h))
+    got = _render(dcmod, ctx, views)
+    pts = np.concatenate([O.pixel_centres(v[:4], v[4], v[5]) for v in views])
+    ref = O.layer_potential(disc, pts, sig, up - um)
+    # 64-bit coordinates and products of them decide the side beyond a few units in the last place
+    keep = np.concatenate([line_distance(disc.seg_xy[np.abs(disc.seg_xy[:, :2] - p[:1]).max(1) < 0.05 * scale], p)
+                           for p in np.split(pts, np.cumsum([v[4] * v[5] for v in views])[:-1])]) > 4 * ulp
+    assert keep.sum() > 0.3 * len(pts)
+    assert np.abs(got - ref)[keep].max() <= 1e-5 * max(1.0, np.abs(ref).max())
