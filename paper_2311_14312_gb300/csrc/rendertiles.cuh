@@ -258,8 +258,8 @@ __device__ __forceinline__ void frame_diff(float ah, float al, float bh, float b
     float h, l;
     diff2(ah, al, bh, bl, h, l);
     const float s = __fadd_rn(h, l);
-    hi = s * iw;
-    lo = __fsub_rn(l, __fsub_rn(s, h)) * iw;
+    hi = __fmul_rn(s, iw);
+    lo = __fmul_rn(__fsub_rn(l, __fsub_rn(s, h)), iw);
 }
 __device__ __forceinline__ Piece load_piece(const EvalArgs32 &a, const Frame &F, int f) {
     Piece p;
@@ -270,7 +270,7 @@ __device__ __forceinline__ Piece load_piece(const EvalArgs32 &a, const Frame &F,
     frame_diff(ph.y, pl.y, F.cyh, F.cyl, F.iw, p.y1h, p.y1l);
     frame_diff(ph.z, pl.z, F.cxh, F.cxl, F.iw, p.x2h, p.x2l);
     frame_diff(ph.w, pl.w, F.cyh, F.cyl, F.iw, p.y2h, p.y2l);
-    p.len = t.plen[i] * F.iw;
+    p.len = __fmul_rn(t.plen[i], F.iw);
     const size_t s3 = 3 * (size_t)t.pseg[i];
     const float wgt = -t.pw[i] * kInv2PiF;
     for (int ch = 0; ch < 3; ++ch) {
@@ -281,23 +281,32 @@ __device__ __forceinline__ Piece load_piece(const EvalArgs32 &a, const Frame &F,
     p.heavy = a.heavy[i] != 0;
     return p;
 }
+// Whether a source is far is decided again wherever it is needed (the
+// samples, the pieces of a list too long to stay staged, the FP64 terms) and
+// has to come out the same each time, or a source at the threshold would be
+// taken twice or not at all: every operation's rounding is written out, since
+// the compiler may fuse a product and a sum in one place and not in another.
+//
 // whether all of the piece is at least the separation away from the centre
 __device__ __forceinline__ bool piece_far(const Piece &p, const Frame &F) {
-    const float dx = p.x2h - p.x1h, dy = p.y2h - p.y1h;
-    const float s = -(p.x1h * dx + p.y1h * dy), l2 = dx * dx + dy * dy;   // foot of the centre, times the length
-    const float k = l2 > 0.f ? fminf(fmaxf(s / l2, 0.f), 1.f) : 0.f;
-    const float x = p.x1h + k * dx, y = p.y1h + k * dy, r = (p.heavy ? kSepBig : kSep) * F.R + 1e-6f * p.len;
-    return x * x + y * y >= r * r;
+    const float dx = __fsub_rn(p.x2h, p.x1h), dy = __fsub_rn(p.y2h, p.y1h);
+    const float s = -__fmaf_rn(p.x1h, dx, __fmul_rn(p.y1h, dy));   // foot of the centre, times the length
+    const float l2 = __fmaf_rn(dx, dx, __fmul_rn(dy, dy));
+    const float k = l2 > 0.f ? fminf(fmaxf(__fdiv_rn(s, l2), 0.f), 1.f) : 0.f;
+    const float x = __fmaf_rn(k, dx, p.x1h), y = __fmaf_rn(k, dy, p.y1h);
+    const float r = __fmaf_rn(1e-6f, p.len, __fmul_rn(p.heavy ? kSepBig : kSep, F.R));
+    return __fmaf_rn(x, x, __fmul_rn(y, y)) >= __fmul_rn(r, r);
 }
 // whether cell src (list-3 entry e of the leaf) is far: its bounding circle
 // at the separation, and the sampled circle outside 1.5 of its widths, where
 // its multipole expansion converges as it does for list 3 itself
 __device__ __forceinline__ bool cell_far(const EvalArgs32 &a, const Frame &F, int e, int src, bool big) {
     const float2 off = a.t.w_off[e];
-    const float dx = F.tx - off.x * F.iw, dy = F.ty - off.y * F.iw;   // centre to centre, in leaf widths
-    const float ws = F.iw / a.t.iw[src];
-    const float d = sqrtf(dx * dx + dy * dy);
-    return d - 0.7072f * ws >= (big ? kSepBig : kSep) * F.R && d >= 1.5f * ws + F.R;
+    // centre to centre, in leaf widths
+    const float dx = __fsub_rn(F.tx, __fmul_rn(off.x, F.iw)), dy = __fsub_rn(F.ty, __fmul_rn(off.y, F.iw));
+    const float ws = __fdiv_rn(F.iw, a.t.iw[src]);
+    const float d = __fsqrt_rn(__fmaf_rn(dx, dx, __fmul_rn(dy, dy)));
+    return __fmaf_rn(-0.7072f, ws, d) >= __fmul_rn(big ? kSepBig : kSep, F.R) && d >= __fmaf_rn(1.5f, ws, F.R);
 }
 
 // A sampled rectangle's pixels come in quads +-x +-y around its centre, one

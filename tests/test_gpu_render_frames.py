@@ -1,6 +1,7 @@
 """The FP32 form's pixel rectangles where their frames are strained: canvases
 far from the origin and in pixel units, where a pixel's side of a curve is
-finer than the (hi, lo) coordinates.  Tolerance: the form's 1e-5 of the
+finer than the (hi, lo) coordinates; sources at the distance that decides
+whether a rectangle samples them.  Tolerance: the form's 1e-5 of the
 field."""
 import dataclasses
 
@@ -8,6 +9,7 @@ import numpy as np
 import pytest
 
 from dc_synth import drawing_by_name, random_node_values
+from dc_synth.drawings import Drawing
 
 pytestmark = pytest.mark.gpu
 
@@ -68,3 +70,33 @@ def test_side_of_a_curve_far_from_the_origin(dcmod, cuda_ok, oracle_mod, scale, 
                            for p in np.split(pts, np.cumsum([v[4] * v[5] for v in views])[:-1])]) > 4 * ulp
     assert keep.sum() > 0.3 * len(pts)
     assert np.abs(got - ref)[keep].max() <= 1e-5 * max(1.0, np.abs(ref).max())
+
+
+def _spokes(centre, radii, length, angles, g=4):
+    """Straight radial curves from the given radii outward, one panel each."""
+    u = np.stack([np.cos(angles), np.sin(angles)], 1)
+    a = centre + radii[:, None] * u
+    ctrl = a[:, None] + (length * np.arange(4) / 3.0)[None, :, None] * u[:, None]
+    n = len(angles)
+    col = np.random.default_rng(5).uniform(0, 1, (n, 2, 2, 3))
+    return Drawing("spokes", ctrl, np.zeros(n, bool), col, np.arange(n + 1, dtype=np.int32), np.zeros(n), g=g,
+                   s_per_panel=5 * g)
+
+
+@pytest.mark.parametrize("sep,scale,n", [(2.5, 3.0, 96), (2.5, 3.0, 10), (5.0, 3e4, 96)])
+def test_sources_at_the_sampling_distance(dcmod, cuda_ok, sep, scale, n):
+    # the rectangle of rows and columns 24 .. 31 of 64: radius 3.5 sqrt(2) pixels about its centre; near
+    # ends at sep radii, off by a few units in the last place of the floats that are compared
+    dx = 1.0 / 64
+    centre = np.array([28 * dx, 28 * dx])
+    near = sep * 3.5 * np.sqrt(2.0) * dx
+    radii = near * (1.0 + (np.arange(n) % 33 - 16) * 2.0 ** -24)
+    d = _spokes(centre, radii, 4 * dx, 0.1 + 2 * np.pi * np.arange(n) / n)
+    got, sig = {}, random_node_values(d.n_nodes, seed=36, scale=scale)
+    for form in ("fmm32", "fmm64"):
+        ctx = dcmod.Context(form=form, g=d.g, s_per_panel=d.s_per_panel, leaf_size=4096, domain=(0.0, 0.0, 1.0, 1.0))
+        ctx.build_drawing(d)
+        ctx.set_density(sig)
+        got[form] = _render(dcmod, ctx, [(0.0, 0.0, 1.0, 1.0, 64, 64)])
+        ctx.close()
+    assert np.abs(got["fmm32"] - got["fmm64"]).max() <= 1e-5 * max(1.0, np.abs(got["fmm64"]).max())
