@@ -44,6 +44,10 @@ constexpr float kMaxRadius = 0.36f, kMaxRadiusBig = 0.18f;   // R in leaf widths
 // coordinate; 17 times that covers the differences and products of cross_ff)
 constexpr float kSideBound = 6e-14f;
 constexpr int kMinSampled = 48;    // rectangles of fewer pixels are evaluated directly
+// and so are those with a radius, in leaf widths, whose square is not a normal
+// float: 1 / R has to be one (such pixels are the same point to FP64 except
+// beside the origin)
+constexpr float kMinRadius = 1e-18f;
 constexpr int kStaged = 64;        // near pieces staged per warp
 constexpr int kWarps = 4;          // warps per block
 constexpr int kBlocksPerSM = 4;    // 128 registers; 3 and 5 blocks measured 3-9% slower
@@ -360,7 +364,7 @@ __device__ __forceinline__ void item(const EvalArgs32 &a, int it, BlockMem &B) {
     F.hy = 0.5f * (tl.nr - 1);
     F.R = sqrtf(F.hx * F.hx * F.dxh * F.dxh + F.hy * F.hy * F.dyh * F.dyh);
     const bool hL = a.hL[leaf] != 0;
-    const bool samp = npx >= kMinSampled && F.R <= (hL ? kMaxRadiusBig : kMaxRadius);
+    const bool samp = npx >= kMinSampled && F.R >= kMinRadius && F.R <= (hL ? kMaxRadiusBig : kMaxRadius);
     const int f0 = t.uf_ptr[leaf], f1 = t.uf_ptr[leaf + 1], w0 = t.w_ptr[leaf], w1 = t.w_ptr[leaf + 1];
     constexpr int kChunk = kWarps * kStaged;
     const bool one = f1 - f0 <= kChunk;   // the near pieces are staged once

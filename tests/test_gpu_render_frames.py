@@ -1,8 +1,8 @@
 """The FP32 form's pixel rectangles where their frames are strained: canvases
 far from the origin and in pixel units, where a pixel's side of a curve is
 finer than the (hi, lo) coordinates; sources at the distance that decides
-whether a rectangle samples them.  Tolerance: the form's 1e-5 of the
-field."""
+whether a rectangle samples them; rectangles so small that their radius
+leaves the float range.  Tolerance: the form's 1e-5 of the field."""
 import dataclasses
 
 import numpy as np
@@ -99,4 +99,23 @@ def test_sources_at_the_sampling_distance(dcmod, cuda_ok, sep, scale, n):
         ctx.set_density(sig)
         got[form] = _render(dcmod, ctx, [(0.0, 0.0, 1.0, 1.0, 64, 64)])
         ctx.close()
+    assert np.abs(got["fmm32"] - got["fmm64"]).max() <= 1e-5 * max(1.0, np.abs(got["fmm64"]).max())
+
+
+@pytest.mark.parametrize("scale", [3.0, 3000.0])   # 3000: large sources, whose polynomial is in FP64
+@pytest.mark.parametrize("size", [1e-18, 1e-21, 1e-24, 1e-30, 1e-44, 1e-60, 1e-300])
+def test_rectangles_below_the_float_range(dcmod, cuda_ok, size, scale):
+    d = drawing_by_name("mixed16")
+    views = [(0.0, 0.0, size, size, 64, 64), (0.0, 0.0, size, 0.5, 64, 9), (0.0, 0.0, 0.4, size, 50, 50),
+             (-size, -size, size, size, 5, 5)]
+    got, sig = {}, None
+    for form in ("fmm32", "fmm64"):
+        ctx = dcmod.Context(form=form, g=d.g, s_per_panel=d.s_per_panel, domain=DOMAIN)
+        ctx.build_drawing(d)
+        if sig is None:
+            sig = random_node_values(ctx.sizes().n_nodes, seed=37, scale=scale)
+        ctx.set_density(sig)
+        got[form] = _render(dcmod, ctx, views)
+        ctx.close()
+    assert np.isfinite(got["fmm64"]).all()
     assert np.abs(got["fmm32"] - got["fmm64"]).max() <= 1e-5 * max(1.0, np.abs(got["fmm64"]).max())
