@@ -67,7 +67,7 @@ struct BlockMem {
     // (pad: lanes that read different pieces hit different banks)
     float4 pc[kWarps * kStaged][5];
     float4 far[kWarps][32][3];    // far pieces being sampled: x1 y1 x2 y2 | len sg012 | mg012
-    float4 cf[kCoefs][2];         // a0 b0 a1 b1 | a2 b2 magnitude -
+    float4 cf[kCoefs][2];         // a0 b0 a1 b1 | a2 b2 - -
     float4 d[kWarps][32];         // the samples less their mean (a copy per warp)
     float2 v[kWarps][32][3];      // the warps' shares of the samples, (hi, lo)
     // rectangles with large far sources: the shares' FP64 terms, the samples
@@ -536,7 +536,6 @@ __device__ __forceinline__ void item(const EvalArgs32 &a, int it, BlockMem &B) {
             cb[1] = fmaf(g.y, w.y, cb[1]);
             cb[2] = fmaf(g.z, w.y, cb[2]);
         }
-        float mag = 0.f;
         for (int ch = 0; ch < 3; ++ch) {
             for (int o = 4; o < 32; o <<= 1) {
                 ca[ch] += __shfl_xor_sync(full, ca[ch], o);
@@ -544,11 +543,10 @@ __device__ __forceinline__ void item(const EvalArgs32 &a, int it, BlockMem &B) {
             }
             ca[ch] *= 2.f / kSamples;
             cb[ch] *= 2.f / kSamples;
-            mag = fmaxf(mag, fabsf(ca[ch]) + fabsf(cb[ch]));
         }
         if (lane < 4) {
             B.cf[k][0] = make_float4(ca[0], cb[0], ca[1], cb[1]);
-            B.cf[k][1] = make_float4(ca[2], cb[2], k == 0 ? 0.f : mag, 0.f);
+            B.cf[k][1] = make_float4(ca[2], cb[2], 0.f, 0.f);
         }
         if (big && warp == 0) {   // FP64 coefficients
             const int k = lane & 15, j0 = lane & 16;
@@ -571,14 +569,25 @@ __device__ __forceinline__ void item(const EvalArgs32 &a, int it, BlockMem &B) {
             }
         }
         __syncthreads();
-        // terms whose sum is below a sixteenth of the FP32 rounding of the value are left out
-        float tail = B.cf[lane & 15][1].z;   // sum over k' >= k
-        for (int o = 1; o < 16; o <<= 1) {
-            const float x = __shfl_down_sync(full, tail, o, 16);
-            if ((lane & 15) + o < 16) tail += x;
+        // Terms whose sum is below a sixteenth of the FP32 rounding of the
+        // value are left out; every channel has its own value, which may be
+        // far smaller than another's.
+        bool need = false;
+        {
+            const float4 c0 = B.cf[lane & 15][0], c1 = B.cf[lane & 15][1];
+            const bool is0 = (lane & 15) == 0;
+            const float mag[3] = {fabsf(c0.x) + fabsf(c0.y), fabsf(c0.z) + fabsf(c0.w), fabsf(c1.x) + fabsf(c1.y)};
+#pragma unroll
+            for (int ch = 0; ch < 3; ++ch) {
+                float tail = is0 ? 0.f : mag[ch];   // sum over k' >= k
+                for (int o = 1; o < 16; o <<= 1) {
+                    const float x = __shfl_down_sync(full, tail, o, 16);
+                    if ((lane & 15) + o < 16) tail += x;
+                }
+                need |= tail > 4e-9f * (__shfl_sync(full, tail, 0) + fabsf(mean[ch]));
+            }
         }
-        const float whole = __shfl_sync(full, tail, 0) + fmaxf(fabsf(mean[0]), fmaxf(fabsf(mean[1]), fabsf(mean[2])));
-        const unsigned keep = __ballot_sync(full, (lane & 15) > 0 && tail > 4e-9f * whole) & 0xffffu;
+        const unsigned keep = __ballot_sync(full, (lane & 15) > 0 && need) & 0xffffu;
         kmax = keep ? 32 - __clz(keep) : 1;
     }
 

@@ -2,7 +2,8 @@
 far from the origin and in pixel units, where a pixel's side of a curve is
 finer than the (hi, lo) coordinates; sources at the distance that decides
 whether a rectangle samples them; rectangles so small that their radius
-leaves the float range.  Tolerance: the form's 1e-5 of the field."""
+leaves the float range; channels of very different size.  Tolerance: the
+form's 1e-5 of the field, 1e-6 between the same form's values."""
 import dataclasses
 
 import numpy as np
@@ -119,3 +120,23 @@ def test_rectangles_below_the_float_range(dcmod, cuda_ok, size, scale):
         ctx.close()
     assert np.isfinite(got["fmm64"]).all()
     assert np.abs(got["fmm32"] - got["fmm64"]).max() <= 1e-5 * max(1.0, np.abs(got["fmm64"]).max())
+
+
+@pytest.mark.parametrize("channel", [0, 2])
+def test_channel_beside_a_large_constant_one(dcmod, cuda_ok, channel):
+    # a channel that is 5 inside the closed curves and 0 outside beside one a million times smaller: what the
+    # small one loses has to be small against itself, so it is compared with its values when it is alone
+    d = drawing_by_name("closed4")
+    u, n = [], d.n_nodes
+    sig = np.zeros((n, 3))
+    sig[:, channel] = 1e-6 * random_node_values(n, seed=38)[:, 0]
+    for jump in (5.0, 0.0):
+        col = np.zeros_like(d.colours)
+        col[:, 0, :, 1] = jump
+        ctx = dcmod.Context(form="fmm32", g=d.g, s_per_panel=d.s_per_panel, domain=DOMAIN)
+        ctx.build_drawing(dataclasses.replace(d, colours=col))
+        ctx.set_density(sig)
+        u.append(_render(dcmod, ctx, [(0.0, 0.0, 1.0, 1.0, 300, 200), (0.3, 0.3, 0.31, 0.32, 128, 96),
+                                      (0.0, 0.0, 1.0, 1.0, 1100, 900)])[:, channel])
+        ctx.close()
+    assert np.abs(u[0] - u[1]).max() <= 1e-6 * np.abs(u[1]).max()
