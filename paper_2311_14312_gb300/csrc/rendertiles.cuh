@@ -84,6 +84,20 @@ __device__ __forceinline__ float2 two_sum(float a, float b) {
     return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
 }
 
+// u + e / 2 pi as a float and its rest: what expansions give is added to what
+// pieces give without rounding, since the two may cancel
+__device__ __forceinline__ float2 add_expansion(float u, float e) {
+    constexpr float kLo = (float)(kInv2Pi - (double)kInv2PiF);
+    const float p = __fmul_rn(e, kInv2PiF);
+    const float2 z = two_sum(u, p);
+    return make_float2(z.x, z.y + fmaf(e, kLo, __fmaf_rn(e, kInv2PiF, -p)));
+}
+// mean + u + e / 2 pi + small, rounded once (but for the small part)
+__device__ __forceinline__ float add_parts(float mean, float u, float e, float small) {
+    const float2 z = add_expansion(u, e), y = two_sum(mean, z.x);
+    return y.x + (y.y + (z.y + small));
+}
+
 // ilog = int log|p - q| and phi = the subtended angle of the segment from a
 // to b (relative to the target q) in closed form (App. D), FP32.  A call,
 // like the FP64 form: the loops that use them would not fit the instruction
@@ -467,9 +481,9 @@ __device__ __forceinline__ void item(const EvalArgs32 &a, int it, BlockMem &B) {
             e2 += w.z;
         }
         float2 *v = B.v[warp][lane];
-        v[0] = two_sum(u0, e0 * kInv2PiF);
-        v[1] = two_sum(u1, e1 * kInv2PiF);
-        v[2] = two_sum(u2, e2 * kInv2PiF);
+        v[0] = add_expansion(u0, e0);
+        v[1] = add_expansion(u1, e1);
+        v[2] = add_expansion(u2, e2);
         if (flags & 1)
             for (int ch = 0; ch < 3; ++ch) B.h[warp][lane][ch] = h[ch];
     } else if (w1 > w0) {
@@ -733,35 +747,42 @@ __device__ __forceinline__ void item(const EvalArgs32 &a, int it, BlockMem &B) {
                     if (one) break;
                 }
             __syncwarp();
-            // expansions at the pixels: the near list-3 cells, and without samples the local one
+            // expansions at the pixels: the near list-3 cells, and without
+            // samples the local one.  They have a sum of their own (times
+            // 2 pi), added to the pieces' at the end: the two may cancel.
+            e0 = e1 = e2 = 0.f;
             if (any_w)
                 for (int k = w0 + sub; k < w1; k += nsub) {
                     const int src = t.w_idx[k];
                     if (a.hM[src] || (samp && cell_far(a, F, k, src, false))) continue;
                     const float3 w = m2p32(a, F, k, src, xh, yh);
-                    u0 = fmaf(w.x, kInv2PiF, u0);
-                    u1 = fmaf(w.y, kInv2PiF, u1);
-                    u2 = fmaf(w.z, kInv2PiF, u2);
+                    e0 += w.x;
+                    e1 += w.y;
+                    e2 += w.z;
                 }
             __syncwarp();
             if (!samp && !hL && sub == nsub - 1) {
                 float2 s0, s1, s2;
                 horner3(a.L + (size_t)leaf * 3 * P1, P1, 0, make_float2(xh + F.tx, yh + F.ty), s0, s1, s2);
-                u0 = fmaf(s0.x, kInv2PiF, u0);
-                u1 = fmaf(s1.x, kInv2PiF, u1);
-                u2 = fmaf(s2.x, kInv2PiF, u2);
+                e0 += s0.x;
+                e1 += s1.x;
+                e2 += s2.x;
             }
             __syncwarp();
             for (int o = ng; o < 32; o <<= 1) {
                 u0 += __shfl_xor_sync(full, u0, o);
                 u1 += __shfl_xor_sync(full, u1, o);
                 u2 += __shfl_xor_sync(full, u2, o);
+                e0 += __shfl_xor_sync(full, e0, o);
+                e1 += __shfl_xor_sync(full, e1, o);
+                e2 += __shfl_xor_sync(full, e2, o);
             }
+            float pv0 = 0.f, pv1 = 0.f, pv2 = 0.f;   // the polynomial less the mean
             if (samp && !big) {
                 const float *pv = &B.pv[warp][3 * slot][quad];
-                u0 = mean[0] + (rest[0] + (u0 + pv[0]));
-                u1 = mean[1] + (rest[1] + (u1 + pv[32]));
-                u2 = mean[2] + (rest[2] + (u2 + pv[64]));
+                pv0 = rest[0] + pv[0];
+                pv1 = rest[1] + pv[32];
+                pv2 = rest[2] + pv[64];
             }
             // FP64 terms
             if (flag64 || big) {
@@ -777,7 +798,6 @@ __device__ __forceinline__ void item(const EvalArgs32 &a, int it, BlockMem &B) {
                         wy = wx * zy + wy * zx;
                         wx = nx;
                     }
-                    for (int ch = 0; ch < 3; ++ch) h[ch] += mean[ch];
                 }
                 if (!samp && hL) add3(h, l2p64(a, leaf, qx64, qy64));
                 if (flag64 && any_w)
@@ -802,9 +822,13 @@ __device__ __forceinline__ void item(const EvalArgs32 &a, int it, BlockMem &B) {
                             add3(h, p2p64(a, __shfl_sync(full, idx, src), qx64, qy64));
                         }
                     }
-                u0 = (float)((double)u0 + h[0]);
-                u1 = (float)((double)u1 + h[1]);
-                u2 = (float)((double)u2 + h[2]);
+                u0 = (float)(((double)u0 + (double)e0 * kInv2Pi) + (h[0] + ((double)mean[0] + pv0)));
+                u1 = (float)(((double)u1 + (double)e1 * kInv2Pi) + (h[1] + ((double)mean[1] + pv1)));
+                u2 = (float)(((double)u2 + (double)e2 * kInv2Pi) + (h[2] + ((double)mean[2] + pv2)));
+            } else {   // without samples the mean is zero
+                u0 = add_parts(mean[0], u0, e0, pv0);
+                u1 = add_parts(mean[1], u1, e1, pv1);
+                u2 = add_parts(mean[2], u2, e2, pv2);
             }
             if (on && sub == 0) {
                 const size_t o = 3 * ((size_t)vp.offset + (size_t)r * vp.width + c);

@@ -2,8 +2,9 @@
 far from the origin and in pixel units, where a pixel's side of a curve is
 finer than the (hi, lo) coordinates; sources at the distance that decides
 whether a rectangle samples them; rectangles so small that their radius
-leaves the float range; channels of very different size.  Tolerance: the
-form's 1e-5 of the field, 1e-6 between the same form's values."""
+leaves the float range; channels of very different size; the mean of a large
+far field.  Tolerance: the form's 1e-5 of the field where none is derived.
+"""
 import dataclasses
 
 import numpy as np
@@ -140,3 +141,26 @@ def test_channel_beside_a_large_constant_one(dcmod, cuda_ok, channel):
                                       (0.0, 0.0, 1.0, 1.0, 1100, 900)])[:, channel])
         ctx.close()
     assert np.abs(u[0] - u[1]).max() <= 1e-6 * np.abs(u[1]).max()
+
+
+@pytest.mark.parametrize("views", [[(0.0, 0.0, 1.0, 1.0, 1100, 900)], [(0.0, 0.0, 1.0, 1.0, 311, 287)],
+                                   [(x / 64, y / 64, (x + 1) / 64, (y + 1) / 64, 6, 7) for x in range(64) for y in range(64)]])
+def test_large_far_field_is_not_biased(dcmod, cuda_ok, views):
+    # 5 inside closed curves, nearly all of it from the expansions.  They are FP32, so a pixel is off by some
+    # 1e-7 of its value and a leaf's mean by 2e-8 (its leading coefficient's rounding); a mean over a hundred
+    # leaves and tens of thousands of pixels is not off by more than a few 1e-9
+    d = drawing_by_name("closed4")
+    col = np.zeros_like(d.colours)
+    col[:, 1] = 5.0
+    got, sig = {}, random_node_values(d.n_nodes, seed=39)
+    for form in ("fmm32", "fmm64"):
+        ctx = dcmod.Context(form=form, g=d.g, s_per_panel=d.s_per_panel, leaf_size=16, domain=DOMAIN)
+        ctx.build_drawing(dataclasses.replace(d, colours=col))
+        ctx.set_density(sig)
+        got[form] = _render(dcmod, ctx, views)
+        ctx.close()
+    big = np.abs(got["fmm64"]) > 3.0
+    assert big.sum() > 10000
+    mean = (got["fmm32"] / got["fmm64"] - 1.0)[big].mean()
+    print(f"mean relative error {mean:.2e} of {big.sum()}")
+    assert abs(mean) <= 1.5e-8
