@@ -547,6 +547,11 @@ dc_status dc_build_tree(dc_ctx *ctx, int n_curves, const double *ctrl, const int
     D.g = G.g;
     D.s = G.s;
     D.n_panels = G.n_panels;
+    for (size_t i = 0; i < G.seg_xy.size(); ++i) {
+        const int d = int(i & 1);
+        D.box[d] = i < 2 ? G.seg_xy[i] : std::min(D.box[d], G.seg_xy[i]);
+        D.box[2 + d] = i < 2 ? G.seg_xy[i] : std::max(D.box[2 + d], G.seg_xy[i]);
+    }
     cudaStream_t s = ctx->stream;
     // buffers of the previous drawing are reused when large enough
     auto up = [&](auto &buf, const auto &vec, const char *what) -> dc_status {

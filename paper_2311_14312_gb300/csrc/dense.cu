@@ -7,6 +7,9 @@
 //  - K12 output conversion / 8-bit quantisation
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
+
 #include "dc_internal.h"
 #include "evalff.cuh"
 #include "segint.cuh"
@@ -156,17 +159,21 @@ __device__ void dense_eval_body(double qx, double qy, bool active, const double 
 // consecutive pixels, kGridSets threads to each, every set its share of the
 // segments (each pixel alone would leave most of the GPU idle below a few
 // hundred thousand pixels); the sets' sums are added in order.  The frame's
-// origin is the middle of the run.  Bound by FP32 issue, 450 instructions a
+// origin is the middle of the run and its unit w, a power of two at least as
+// large as the drawing and the viewport, so that squares of distances are
+// normal floats on any canvas; the logarithms are then log(r / w), and log(w)
+// times the segments' weighted lengths is added in FP64.  Bound by FP32 issue, 450 instructions a
 // pair: 128^2 pixels of 5,120 segments in 1.86 ms on one GB300, 27.7 with the
 // pairs in FP64.
 constexpr int kGridPixels = 64, kGridSets = 4;
 __global__ void __launch_bounds__(kGridPixels *kGridSets, 2)
 dense_eval_grid_kernel(const double *__restrict__ seg, const double *__restrict__ segw,
                        const double *__restrict__ sbar, const double *__restrict__ mbar, int S,
-                       VpDev vp, double *__restrict__ u) {
+                       VpDev vp, double w, double *__restrict__ u) {
     __shared__ ff::Tables T;
     __shared__ evalff::Stage t[kGridSets];
     __shared__ double red[kGridSets - 1][3][kGridPixels];
+    __shared__ double red3[kGridPixels * kGridSets / 32][3];
     ff::init_tables(T);
     const long long npix = (long long)vp.width * vp.height;
     const long long first = (long long)blockIdx.x * kGridPixels;
@@ -180,7 +187,9 @@ dense_eval_grid_kernel(const double *__restrict__ seg, const double *__restrict_
     double cx, cy, qx, qy;
     centre(min(first + kGridPixels / 2, npix - 1), cx, cy);
     centre(pix, qx, qy);
-    const float2 x = ff::from(qx - cx), y = ff::from(qy - cy);
+    const double iw = 1.0 / w;   // exact
+    const float2 x = ff::from((qx - cx) * iw), y = ff::from((qy - cy) * iw);
+    double k3[3] = {0.0, 0.0, 0.0};   // weighted lengths of the segments this thread staged
     evalff::Sum3 a;
     a.zero();
     constexpr int kRound = evalff::kStage * kGridSets;
@@ -189,9 +198,10 @@ dense_eval_grid_kernel(const double *__restrict__ seg, const double *__restrict_
         const int k = base + threadIdx.x;   // kRound threads: set `set` stages its own share
         if (k < S) {
             const double *q = seg + 4 * (size_t)k;
-            const double dx = q[2] - q[0], dy = q[3] - q[1], w = -segw[k] * kInv2Pi;
-            evalff::stage_segment(t[set], px, q, cx, cy, 1.f, sqrt(dx * dx + dy * dy), w, w, sbar + 3 * (size_t)k,
+            const double dx = q[2] - q[0], dy = q[3] - q[1], wg = -segw[k] * kInv2Pi, len = sqrt(dx * dx + dy * dy);
+            evalff::stage_segment(t[set], px, q, cx, cy, iw, len, wg * w, wg, sbar + 3 * (size_t)k,
                                   mbar + 3 * (size_t)k);
+            for (int c = 0; c < 3; ++c) k3[c] += wg * len * sbar[3 * (size_t)k + c];
         }
         __syncthreads();
         const int cnt = min(evalff::kStage, S - base - set * evalff::kStage);
@@ -200,10 +210,16 @@ dense_eval_grid_kernel(const double *__restrict__ seg, const double *__restrict_
     }
     if (set > 0)
         for (int c = 0; c < 3; ++c) red[set - 1][c][px] = a.v[c];
+    for (int c = 0; c < 3; ++c) {
+        for (int o = 16; o > 0; o >>= 1) k3[c] += __shfl_xor_sync(0xffffffffu, k3[c], o);
+        if ((threadIdx.x & 31) == 0) red3[threadIdx.x >> 5][c] = k3[c];
+    }
     __syncthreads();
     if (set == 0 && first + px < npix)
         for (int c = 0; c < 3; ++c) {
-            double v = a.v[c];
+            double lw = 0.0;
+            for (int i = 0; i < kGridPixels * kGridSets / 32; ++i) lw += red3[i][c];
+            double v = a.v[c] + lw * log(w);
             for (int i = 0; i < kGridSets - 1; ++i) v += red[i][c][px];
             u[3 * pix + c] = v;
         }
@@ -459,9 +475,15 @@ cudaError_t launch_dense_eval_grid(const DevGeom &G, const double *sbar, const d
                                    const VpDev &vp, double *u, cudaStream_t st) {
     long long npix = (long long)vp.width * vp.height;
     if (npix == 0) return cudaSuccess;
+    double ext = 0.0;   // of the segments and the viewport
+    for (int d = 0; d < 2; ++d) {
+        const double a = d ? vp.y0 : vp.x0, b = a + (d ? vp.height * vp.dy : vp.width * vp.dx);
+        ext = std::max(ext, std::max({G.box[2 + d], a, b}) - std::min({G.box[d], a, b}));
+    }
+    const double w = std::ldexp(1.0, ext > 0.0 && std::isfinite(ext) ? std::min(std::ilogb(ext) + 1, 1000) : 0);
     unsigned blocks = (unsigned)((npix + kGridPixels - 1) / kGridPixels);
-    dense_eval_grid_kernel<<<blocks, kGridPixels * kGridSets, 0, st>>>(G.seg.ptr, G.segw.ptr, sbar, mbar, G.S,
-                                                            vp, u); note_launch();
+    dense_eval_grid_kernel<<<blocks, kGridPixels * kGridSets, 0, st>>>(G.seg.ptr, G.segw.ptr, sbar, mbar, G.S, vp, w,
+                                                                    u); note_launch();
     return cudaGetLastError();
 }
 

@@ -21,17 +21,18 @@ struct Stage {
 };
 
 // Entry i of the stage: the segment q (x1 y1 x2 y2) relative to (cx, cy),
-// times iw (a power of two); ks, km: what multiplies sb and mb.
+// times iw (a power of two that brings the frame to about one: squares of
+// distances have to stay normal floats); ks, km: what multiplies sb and mb.
 __device__ __forceinline__ void stage_segment(Stage &t, int i, const double *__restrict__ q, double cx, double cy,
-                                              float iw, double len, double ks, double km,
+                                              double iw, double len, double ks, double km,
                                               const double *__restrict__ sb, const double *__restrict__ mb) {
-    const float2 x1 = ff::scale(ff::from(q[0] - cx), iw), y1 = ff::scale(ff::from(q[1] - cy), iw);
-    const float2 x2 = ff::scale(ff::from(q[2] - cx), iw), y2 = ff::scale(ff::from(q[3] - cy), iw);
-    const float2 dx = ff::scale(ff::from(q[2] - q[0]), iw), dy = ff::scale(ff::from(q[3] - q[1]), iw);
+    const float2 x1 = ff::from((q[0] - cx) * iw), y1 = ff::from((q[1] - cy) * iw);
+    const float2 x2 = ff::from((q[2] - cx) * iw), y2 = ff::from((q[3] - cy) * iw);
+    const float2 dx = ff::from((q[2] - q[0]) * iw), dy = ff::from((q[3] - q[1]) * iw);
     t.p1[i] = make_float4(x1.x, x1.y, y1.x, y1.y);
     t.p2[i] = make_float4(x2.x, x2.y, y2.x, y2.y);
     t.d[i] = make_float4(dx.x, dx.y, dy.x, dy.y);
-    t.len[i] = ff::scale(ff::from(len), iw);
+    t.len[i] = ff::from(len * iw);
     for (int c = 0; c < 3; ++c) {
         t.sg[i][c] = ff::from(ks * sb[c]);
         t.mg[i][c] = ff::from(km * mb[c]);

@@ -132,7 +132,8 @@ __device__ __forceinline__ float2 atan2(const Tables &T, float2 y, float2 x) {
     const bool sw = y.x > x.x;
     const float2 n = sw ? x : y, d = sw ? y : x;
     // t = n / d in [0, 1]; atan t = atan t_k + atan((n - t_k d) / (d + t_k n)), t_k = k / 16
-    const int k = __float2int_rn(16.f * __fdividef(n.x, d.x));
+    // (at most 16 by rounding; the bound holds for arguments out of range too, denormal ones among them)
+    const int k = min(max(__float2int_rn(16.f * __fdividef(n.x, d.x)), 0), kAtanEntries - 1);
     const float tk = (float)k * 0.0625f;
     const float2 num = sub(n, mulf(d, tk)), den = add(d, mulf(n, tk));
     const float2 v = mul(num, inv(den));   // |v| <= 1/32

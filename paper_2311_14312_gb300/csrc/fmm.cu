@@ -88,11 +88,11 @@ eval_tiles_kernel(DevTree t, const RTile *__restrict__ tiles, int n_tiles, int *
         const VpDev &vp = vps[tl.vp];
         const int leaf = tl.leaf, npx = tl.nr * tl.nc, j = threadIdx.x;
         const double cx = t.cc[2 * leaf], cy = t.cc[2 * leaf + 1], w = t.cw[leaf];
-        const float iw = (float)(1.0 / w);   // exact: a power of two
+        const double iw = 1.0 / w;   // exact: a power of two
         const bool on = j < npx;
         const int r = tl.r0 + (on ? j / tl.nc : 0), c = tl.c0 + (on ? j % tl.nc : 0);
-        const float2 x = ff::scale(ff::from(vp.x0 + (c + 0.5) * vp.dx - cx), iw);
-        const float2 y = ff::scale(ff::from(vp.y0 + (r + 0.5) * vp.dy - cy), iw);
+        const float2 x = ff::from((vp.x0 + (c + 0.5) * vp.dx - cx) * iw);
+        const float2 y = ff::from((vp.y0 + (r + 0.5) * vp.dy - cy) * iw);
         evalff::Sum3 u, e;   // list 1; expansions, times 2 pi
         u.zero();
         e.zero();
