@@ -547,10 +547,15 @@ dc_status dc_build_tree(dc_ctx *ctx, int n_curves, const double *ctrl, const int
     D.g = G.g;
     D.s = G.s;
     D.n_panels = G.n_panels;
-    for (size_t i = 0; i < G.seg_xy.size(); ++i) {
-        const int d = int(i & 1);
-        D.box[d] = i < 2 ? G.seg_xy[i] : std::min(D.box[d], G.seg_xy[i]);
-        D.box[2 + d] = i < 2 ? G.seg_xy[i] : std::max(D.box[2 + d], G.seg_xy[i]);
+    if (ctx->opt.form == DC_FORM_DENSE64 && !G.seg_xy.empty()) {   // its pixel frames' unit
+        double x0 = G.seg_xy[0], x1 = x0, y0 = G.seg_xy[1], y1 = y0;
+        for (size_t i = 0; i < G.seg_xy.size(); i += 2) {
+            x0 = std::min(x0, G.seg_xy[i]);
+            x1 = std::max(x1, G.seg_xy[i]);
+            y0 = std::min(y0, G.seg_xy[i + 1]);
+            y1 = std::max(y1, G.seg_xy[i + 1]);
+        }
+        D.box[0] = x0, D.box[1] = y0, D.box[2] = x1, D.box[3] = y1;
     }
     cudaStream_t s = ctx->stream;
     // buffers of the previous drawing are reused when large enough

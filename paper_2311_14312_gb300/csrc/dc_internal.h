@@ -157,7 +157,7 @@ struct DevBuf {
 // Device copy of the discretisation.
 struct DevGeom {
     int N = 0, S = 0, g = 0, s = 0, n_panels = 0;
-    double box[4] = {0.0, 0.0, 0.0, 0.0};   // x0 y0 x1 y1 around the segments
+    double box[4] = {0.0, 0.0, 0.0, 0.0};   // x0 y0 x1 y1 around the segments (dense form)
     DevBuf<double> seg;       // [S][4]
     DevBuf<double> segw;      // [S]
     DevBuf<double> node_xy;   // [N][2]
