@@ -188,7 +188,7 @@ dense_eval_grid_kernel(const double *__restrict__ seg, const double *__restrict_
     centre(min(first + kGridPixels / 2, npix - 1), cx, cy);
     centre(pix, qx, qy);
     const double iw = 1.0 / w;   // exact
-    const float2 x = ff::from((qx - cx) * iw), y = ff::from((qy - cy) * iw);
+    const ff::Coord x = ff::coord((qx - cx) * iw), y = ff::coord((qy - cy) * iw);
     double k3[3] = {0.0, 0.0, 0.0};   // weighted lengths of the segments this thread staged
     evalff::Sum3 a;
     a.zero();
@@ -205,7 +205,9 @@ dense_eval_grid_kernel(const double *__restrict__ seg, const double *__restrict_
         }
         __syncthreads();
         const int cnt = min(evalff::kStage, S - base - set * evalff::kStage);
-        for (int i = 0; i < cnt; ++i) evalff::add_segment(T, t[set], i, x, y, a);
+        const double *own = seg + 4 * (size_t)(base + set * evalff::kStage);
+        for (int i = 0; i < cnt; ++i)
+            evalff::add_segment(T, t[set], i, x, y, a, [&] { return evalff::cross64(own + 4 * i, qx, qy) * iw * iw; });
         a.flush();
     }
     if (set > 0)

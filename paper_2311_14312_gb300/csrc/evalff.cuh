@@ -15,8 +15,8 @@ constexpr int kStage = 64;   // segments staged per round
 
 struct Stage {
     // x1 y1 | x2 y2 | dx dy, each (hi, lo); len and the weights of the three
-    // channels: -w sigma / 2 pi and -w mu / 2 pi
-    float4 p1[kStage], p2[kStage], d[kStage];
+    // channels: -w sigma / 2 pi and -w mu / 2 pi; p3: third floats of x1 y1 x2 y2
+    float4 p1[kStage], p2[kStage], p3[kStage], d[kStage];
     float2 len[kStage], sg[kStage][3], mg[kStage][3];
 };
 
@@ -26,11 +26,12 @@ struct Stage {
 __device__ __forceinline__ void stage_segment(Stage &t, int i, const double *__restrict__ q, double cx, double cy,
                                               double iw, double len, double ks, double km,
                                               const double *__restrict__ sb, const double *__restrict__ mb) {
-    const float2 x1 = ff::from((q[0] - cx) * iw), y1 = ff::from((q[1] - cy) * iw);
-    const float2 x2 = ff::from((q[2] - cx) * iw), y2 = ff::from((q[3] - cy) * iw);
+    const ff::Coord x1 = ff::coord((q[0] - cx) * iw), y1 = ff::coord((q[1] - cy) * iw);
+    const ff::Coord x2 = ff::coord((q[2] - cx) * iw), y2 = ff::coord((q[3] - cy) * iw);
     const float2 dx = ff::from((q[2] - q[0]) * iw), dy = ff::from((q[3] - q[1]) * iw);
-    t.p1[i] = make_float4(x1.x, x1.y, y1.x, y1.y);
-    t.p2[i] = make_float4(x2.x, x2.y, y2.x, y2.y);
+    t.p1[i] = make_float4(x1.f.x, x1.f.y, y1.f.x, y1.f.y);
+    t.p2[i] = make_float4(x2.f.x, x2.f.y, y2.f.x, y2.f.y);
+    t.p3[i] = make_float4(x1.t, y1.t, x2.t, y2.t);
     t.d[i] = make_float4(dx.x, dx.y, dy.x, dy.y);
     t.len[i] = ff::from(len * iw);
     for (int c = 0; c < 3; ++c) {
@@ -59,13 +60,39 @@ struct Sum3 {
         }
     }
 };
-// u += entry i's single and double layer at the target (x, y) of the frame
-__device__ __forceinline__ void add_segment(const ff::Tables &T, const Stage &t, int i, float2 x, float2 y, Sum3 &u) {
+// a x b of the segment P (x1 y1 x2 y2) at the target (qx, qy), in FP64
+static __device__ __noinline__ double cross64(const double *__restrict__ P, double qx, double qy) {
+    return (P[0] - qx) * (P[3] - qy) - (P[1] - qy) * (P[2] - qx);
+}
+// what ff::pair asks of a pair's coordinates, from two lambdas
+template <typename R, typename C>
+struct NearPair {
+    R refine;
+    C cross;
+};
+template <typename R, typename C>
+__device__ __forceinline__ NearPair<R, C> near_pair(R refine, C cross) {
+    return {refine, cross};
+}
+// u += entry i's single and double layer at the target (x, y) of the frame;
+// cross(): the entry's a x b at the target in FP64, in the frame's unit
+template <typename Cross>
+__device__ __forceinline__ void add_segment(const ff::Tables &T, const Stage &t, int i, ff::Coord x, ff::Coord y, Sum3 &u,
+                                            const Cross &cross) {
     const float4 p1 = t.p1[i], p2 = t.p2[i], d = t.d[i];
     float2 il, ph;
-    ff::pair(T, ff::sub(make_float2(p1.x, p1.y), x), ff::sub(make_float2(p1.z, p1.w), y),
-             ff::sub(make_float2(p2.x, p2.y), x), ff::sub(make_float2(p2.z, p2.w), y), make_float2(d.x, d.y),
-             make_float2(d.z, d.w), t.len[i], il, ph);
+    const auto near = near_pair(
+        [&](float2 &ax, float2 &ay, float2 &bx, float2 &by) {
+            const float4 p3 = t.p3[i];
+            ax = ff::diff({make_float2(p1.x, p1.y), p3.x}, x);
+            ay = ff::diff({make_float2(p1.z, p1.w), p3.y}, y);
+            bx = ff::diff({make_float2(p2.x, p2.y), p3.z}, x);
+            by = ff::diff({make_float2(p2.z, p2.w), p3.w}, y);
+        },
+        cross);
+    ff::pair(T, ff::sub(make_float2(p1.x, p1.y), x.f), ff::sub(make_float2(p1.z, p1.w), y.f),
+             ff::sub(make_float2(p2.x, p2.y), x.f), ff::sub(make_float2(p2.z, p2.w), y.f), make_float2(d.x, d.y),
+             make_float2(d.z, d.w), t.len[i], il, ph, false, near);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         dot2ff(u.h[c], u.l[c], il, t.sg[i][c]);

@@ -12,7 +12,7 @@
 
 #include <cuda_runtime.h>
 
-#include "ffmath.cuh"
+#include "evalff.cuh"
 #include "passes.cuh"
 
 namespace dc {
@@ -292,11 +292,8 @@ static __global__ void __launch_bounds__(32 * kWarps) near_coef_kernel(NodeArgs<
 // The build of a 200-curve drawing takes 11.1 ms instead of 12.7, curves to
 // image 21.7 instead of 24.2.
 constexpr int kFfLeaf = 256;
-__device__ __forceinline__ float ff_rest(double v, float2 f) { return (float)((v - (double)f.x) - (double)f.y); }
-// (a + at) - (b + bt)
-__device__ __forceinline__ float2 ff_diff(float2 a, float at, float2 b, float bt) {
-    return ff::addf(ff::sub(a, b), at - bt);
-}
+// a - b for pairs that are not near, where the rounding of the lo parts' difference does not show
+__device__ __forceinline__ float2 ff_diff(ff::Coord a, ff::Coord b) { return ff::addf(ff::sub(a.f, b.f), a.t - b.t); }
 static __global__ void __launch_bounds__(32 * kWarps) near_coef_ff_kernel(NodeArgs<double> a,
                                                                     const long long *__restrict__ off, int n_items,
                                                                     float2 *__restrict__ cg, float2 *__restrict__ cf,
@@ -306,6 +303,8 @@ static __global__ void __launch_bounds__(32 * kWarps) near_coef_ff_kernel(NodeAr
         swg[kStageN];
     __shared__ float4 st[kStageN];   // the third floats of x1, y1, x2, y2
     __shared__ int sseg[kStageN];
+    __shared__ ff::Coord sqx[kNodeItem], sqy[kNodeItem];   // the item's nodes and their own segments
+    __shared__ int2 sown[kNodeItem];
     ff::init_tables(T);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
@@ -313,20 +312,12 @@ static __global__ void __launch_bounds__(32 * kWarps) near_coef_ff_kernel(NodeAr
         const int leaf = it.x, t0 = it.y, nt = it.z, nU = it.w;
         const long long base = off[item];
         const double cx = a.cc64[2 * leaf], cy = a.cc64[2 * leaf + 1];
-        float2 qx[kPer], qy[kPer];
-        float qxt[kPer], qyt[kPer];
-        int o1[kPer], o2[kPer];
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const int ti = t0 + warp + kWarps * j;
-            const bool ok = (warp + kWarps * j) < nt;
-            const double x = ok ? a.q64[2 * ti] - cx : 0.0, y = ok ? a.q64[2 * ti + 1] - cy : 0.0;
-            qx[j] = ff::from(x);
-            qy[j] = ff::from(y);
-            qxt[j] = ff_rest(x, qx[j]);
-            qyt[j] = ff_rest(y, qy[j]);
-            o1[j] = (ok && a.own1) ? a.own1[ti] : -1;
-            o2[j] = (ok && a.own2) ? a.own2[ti] : -1;
+        __syncthreads();   // the last item's nodes have been read
+        if (threadIdx.x < nt) {
+            const int ti = t0 + threadIdx.x;
+            sqx[threadIdx.x] = ff::coord(a.q64[2 * ti] - cx);
+            sqy[threadIdx.x] = ff::coord(a.q64[2 * ti + 1] - cy);
+            sown[threadIdx.x] = make_int2(a.own1 ? a.own1[ti] : -1, a.own2 ? a.own2[ti] : -1);
         }
         int pl0 = 0;
         for (int e = a.u_ptr[leaf]; e < a.u_ptr[leaf + 1]; ++e) {
@@ -339,12 +330,13 @@ static __global__ void __launch_bounds__(32 * kWarps) near_coef_ff_kernel(NodeAr
                     const int i = p0 + b + s;
                     const double *P = a.pc64 + 4 * (size_t)i;
                     const double dx = P[2] - P[0], dy = P[3] - P[1];
-                    const double x1 = P[0] - cx, y1 = P[1] - cy, x2 = P[2] - cx, y2 = P[3] - cy;
-                    sx1[s] = ff::from(x1);
-                    sy1[s] = ff::from(y1);
-                    sx2[s] = ff::from(x2);
-                    sy2[s] = ff::from(y2);
-                    st[s] = make_float4(ff_rest(x1, sx1[s]), ff_rest(y1, sy1[s]), ff_rest(x2, sx2[s]), ff_rest(y2, sy2[s]));
+                    const ff::Coord x1 = ff::coord(P[0] - cx), y1 = ff::coord(P[1] - cy);
+                    const ff::Coord x2 = ff::coord(P[2] - cx), y2 = ff::coord(P[3] - cy);
+                    sx1[s] = x1.f;
+                    sy1[s] = y1.f;
+                    sx2[s] = x2.f;
+                    sy2[s] = y2.f;
+                    st[s] = make_float4(x1.t, y1.t, x2.t, y2.t);
                     sdx[s] = ff::from(dx);
                     sdy[s] = ff::from(dy);
                     sl[s] = ff::from(sqrt(dx * dx + dy * dy));
@@ -359,10 +351,25 @@ static __global__ void __launch_bounds__(32 * kWarps) near_coef_ff_kernel(NodeAr
                         const int tl = warp + kWarps * j;
                         if (tl >= nt) break;
                         float2 il, phi;
+                        const ff::Coord qx = sqx[tl], qy = sqy[tl];
+                        const int2 o = sown[tl];
+                        auto at = [&](const float2 *v, float t) { return ff::Coord{v[s], t}; };
+                        const auto near = evalff::near_pair(
+                            [&](float2 &ax, float2 &ay, float2 &bx, float2 &by) {
+                                const float4 r = st[s];
+                                ax = ff::diff(at(sx1, r.x), qx);
+                                ay = ff::diff(at(sy1, r.y), qy);
+                                bx = ff::diff(at(sx2, r.z), qx);
+                                by = ff::diff(at(sy2, r.w), qy);
+                            },
+                            [&] {
+                                const double *q = a.q64 + 2 * (size_t)(t0 + tl);
+                                return evalff::cross64(a.pc64 + 4 * (size_t)(p0 + b + s), q[0], q[1]);
+                            });
                         const float4 r = st[s];
-                        ff::pair(T, ff_diff(sx1[s], r.x, qx[j], qxt[j]), ff_diff(sy1[s], r.y, qy[j], qyt[j]),
-                                 ff_diff(sx2[s], r.z, qx[j], qxt[j]), ff_diff(sy2[s], r.w, qy[j], qyt[j]), sdx[s],
-                                 sdy[s], sl[s], il, phi, seg == o1[j] || seg == o2[j]);
+                        ff::pair(T, ff_diff(at(sx1, r.x), qx), ff_diff(at(sy1, r.y), qy), ff_diff(at(sx2, r.z), qx),
+                                 ff_diff(at(sy2, r.w), qy), sdx[s], sdy[s], sl[s], il, phi,
+                                 seg == o.x || seg == o.y, near);
                         const long long idx = base + (long long)tl * nU + pl0 + s;
                         const float2 g = ff::mul(il, swg[s]);
                         cg[idx] = g;

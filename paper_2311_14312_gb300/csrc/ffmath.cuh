@@ -4,8 +4,10 @@
 // 60 other operations) takes the FP64 pipe as long as 18,000 FP32
 // instructions per lane would, the same pair here about 450.  Coordinates
 // are relative to a centre near the targets (the difference is taken in FP64
-// once per piece, not per pair), so that 48 bits of them are more than 53 of
-// the canvas's.  Over 5,120 segments of four closed curves, densities up to
+// once per piece, not per pair).  Where that centre's frame is more than about
+// a thirty-second of the canvas, 48 bits of them are fewer than FP64 has: near
+// pairs take the differences from three floats (Coord), and a target beside a
+// segment takes its side from FP64.  Over 5,120 segments of four closed curves, densities up to
 // 6,000, the pairs add up to 4.4e-15 of the field (the series beyond four
 // lengths avoids the cancellation of the two logarithms); in FP64 to 1.9e-13.
 //
@@ -147,12 +149,40 @@ __device__ __forceinline__ float2 atan2(const Tables &T, float2 y, float2 x) {
     return sy ? neg(a) : a;
 }
 
+// A coordinate of the frame as three floats: (hi, lo) drops up to five of a
+// double's bits where the frame is as wide as the canvas, the third holds them.
+struct Coord {
+    float2 f;
+    float t;
+};
+__device__ __forceinline__ Coord coord(double v) {
+    Coord c;
+    c.f = from(v);
+    c.t = (float)((v - (double)c.f.x) - (double)c.f.y);
+    return c;
+}
+// a - b to float-float accuracy of the difference itself, however close the
+// two are: the hi and the lo parts are each subtracted without rounding
+__device__ __forceinline__ float2 diff(Coord a, Coord b) {
+    const float2 s = two_sum(a.f.x, -b.f.x), t = two_sum(a.f.y, -b.f.y), z = two_sum(s.x, t.x);
+    return quick(z.x, __fadd_rn(z.y, __fadd_rn(s.y, __fadd_rn(t.y, __fsub_rn(a.t, b.t)))));
+}
+
 // ilog = int log|p - q| dS and phi = the subtended angle of the segment from
 // a to b (relative to the target), half length vector not needed: d = b - a
 // and len = |d| are the piece's own.  own: the target is a node of the piece's
 // segment, phi = 0.
+// Within four lengths the angle takes what a and b lose to (hi, lo)
+// coordinates over the distance: near.refine(ax, ay, bx, by) then gives them
+// from all bits (56 instructions more: the plain form's 517 x 509 pixels take
+// 1,048 us instead of 1,014; beyond, what is lost stays below the pair's own
+// rounding).
+// A target beside the segment by less than 2^-40 of it, where rounding could
+// give the wrong side, takes a x b from near.cross(), formed in FP64.
+constexpr float kSide = 0x1p-40f;
+template <typename Near>
 __device__ __forceinline__ void pair(const Tables &T, float2 ax, float2 ay, float2 bx, float2 by, float2 dx, float2 dy,
-                                     float2 len, float2 &ilog, float2 &phi, bool own = false) {
+                                     float2 len, float2 &ilog, float2 &phi, bool own, const Near &near) {
     const float2 mx = scale(add(ax, bx), 0.5f), my = scale(add(ay, by), 0.5f);   // midpoint
     const float2 r2 = dot(mx, mx, my, my);
     if (!own && 16.f * len.x * len.x < r2.x) {
@@ -193,7 +223,11 @@ __device__ __forceinline__ void pair(const Tables &T, float2 ax, float2 ay, floa
         phi = scale(dot(ex, wy, ey, wx), 2.f);
         return;
     }
-    const float2 cr = dot(ax, by, neg(ay), bx), dt = dot(ax, bx, ay, by);
+    near.refine(ax, ay, bx, by);
+    float2 cr = dot(ax, by, neg(ay), bx);
+    const float2 dt = dot(ax, bx, ay, by);
+    if (!own && dt.x < 0.f && fabsf(cr.x) < kSide * fmaf(fabsf(ax.x), fabsf(by.x), fabsf(ay.x * bx.x)))
+        cr = from(near.cross());
     phi = own || (cr.x == 0.f && dt.x == 0.f) ? make_float2(0.f, 0.f) : atan2(T, cr, dt);   // own, or at an end point: 0
     const float2 ra2 = dot(ax, ax, ay, ay), rb2 = dot(bx, bx, by, by), il = inv(len);
     const float2 s1 = mul(dot(ax, dx, ay, dy), il), s2 = mul(dot(bx, dx, by, dy), il);

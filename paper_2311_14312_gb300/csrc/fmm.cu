@@ -91,8 +91,9 @@ eval_tiles_kernel(DevTree t, const RTile *__restrict__ tiles, int n_tiles, int *
         const double iw = 1.0 / w;   // exact: a power of two
         const bool on = j < npx;
         const int r = tl.r0 + (on ? j / tl.nc : 0), c = tl.c0 + (on ? j % tl.nc : 0);
-        const float2 x = ff::from((vp.x0 + (c + 0.5) * vp.dx - cx) * iw);
-        const float2 y = ff::from((vp.y0 + (r + 0.5) * vp.dy - cy) * iw);
+        const ff::Coord x3 = ff::coord((vp.x0 + (c + 0.5) * vp.dx - cx) * iw);
+        const ff::Coord y3 = ff::coord((vp.y0 + (r + 0.5) * vp.dy - cy) * iw);
+        const float2 x = x3.f, y = y3.f;
         evalff::Sum3 u, e;   // list 1; expansions, times 2 pi
         u.zero();
         e.zero();
@@ -160,7 +161,11 @@ eval_tiles_kernel(DevTree t, const RTile *__restrict__ tiles, int n_tiles, int *
             }
             __syncthreads();
             if (on)
-                for (int i = 0; i < n; ++i) evalff::add_segment(T, S, i, x, y, u);
+                for (int i = 0; i < n; ++i)
+                    evalff::add_segment(T, S, i, x3, y3, u, [&] {
+                        return evalff::cross64(t.pc + 4 * (size_t)uf_idx[f0 + i], vp.x0 + (c + 0.5) * vp.dx,
+                                               vp.y0 + (r + 0.5) * vp.dy) * iw * iw;
+                    });
             u.flush();
         }
         for (int ch = 0; ch < 3; ++ch) {
