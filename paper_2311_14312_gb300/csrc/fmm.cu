@@ -571,13 +571,16 @@ cudaError_t Fmm::Impl::build_near(cudaStream_t st) {
     if (fp32 && (e = near_g32.alloc((size_t)near_total)) != cudaSuccess) return e;
     // The FP64 node operator reads near and far coefficients in float-float
     // when both are stored; the near ones are then formed so at once.  Not with
-    // large leaves (near_coef_ff_kernel says why), nor on a canvas so small
+    // large leaves (near_coef_ff_kernel says why; the depth limit can leave
+    // any number of pieces in one, whatever leaf_size), nor on a canvas so small
     // that the square of a coordinate's last bit leaves the floats' range, or
     // so large that a squared distance might: FP64, narrowed.
     const size_t need_far = (size_t)far_blocks * (P1 * sizeof(double2) + (fp32 ? P1i * sizeof(float2) : 0));
     const bool want_far = far_blocks > 0 && need_far <= (fr - need) / 4;
-    const bool ff_direct =
-        want_far && opt.leaf_size <= evalnodes::kFfLeaf && tree.w0 >= 0x1p-7 && tree.w0 <= 0x1p20;
+    int most = 0;   // pieces of a leaf
+    for (int c = 0; c < tree.n_cells(); ++c)
+        if (tree.is_leaf(c)) most = std::max(most, tree.piece_count[c]);
+    const bool ff_direct = want_far && most <= evalnodes::kFfLeaf && tree.w0 >= 0x1p-7 && tree.w0 <= 0x1p20;
     evalnodes::NodeArgs<double> a = node_args64(nt_items4.ptr, nt_xy.ptr, nt_own1.ptr, nt_own2.ptr,
                                                 nt_perm.ptr, nullptr, nullptr, 0, 0, nullptr);
     if (want_far && ((e = near_gff.alloc((size_t)near_total)) != cudaSuccess ||

@@ -1,7 +1,8 @@
-"""The FP64 forms' float-float pixels where their frames are strained:
-targets 1e-16 to 1e-12 off a curve while the frame is as wide as the canvas,
-and canvases far outside the float range of a squared distance, against the
-oracle's direct sum.  Tolerance: 1e-11 of the field, the FP64 forms' own."""
+"""The FP64 forms' float-float pixels and coefficients where their frames are
+strained: targets 1e-16 to 1e-12 off a curve while the frame is as wide as
+the canvas, canvases far outside the float range of a squared distance, and
+leaves that stop at the depth limit with thousands of pieces.  Tolerance:
+1e-11 of the field, the FP64 forms' own."""
 import dataclasses
 
 import numpy as np
@@ -79,3 +80,23 @@ def test_canvas_outside_the_float_range(dcmod, cuda_ok, oracle_mod, form, e):
     pts = np.concatenate([O.pixel_centres(v[:4], v[4], v[5]) for v in views])
     ref = O.layer_potential(disc, pts, sig, up - um)
     assert np.abs(got - ref).max() <= 1e-11 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("depth", [1, 2, 40])
+def test_operator_with_leaves_at_the_depth_limit(dcmod, cuda_ok, oracle_mod, depth):
+    import torch
+    d = drawing_by_name("mixed16")
+    disc = library_discretisation(dcmod, oracle_mod, d)
+    rows = oracle_mod.hybrid_rows(disc)
+    ctx = dcmod.Context(form="fmm64", g=d.g, s_per_panel=d.s_per_panel, p=30, max_depth=depth, domain=(0.0, 0.0, 1.0, 1.0))
+    ctx.build_drawing(d)
+    v = random_node_values(disc.n_nodes, seed=71)
+    x = torch.from_numpy(v).cuda()
+    y = torch.empty_like(x)
+    for op in (0, 1):
+        ctx.apply_operator(x, y, op)
+        torch.cuda.synchronize()
+        ref = rows[op] @ v
+        err = np.abs(y.cpu().numpy() - ref).max() / np.abs(ref).max()
+        print(f"depth {depth} op {op}: {err:.2e}")
+        assert err <= 1e-11
