@@ -53,7 +53,8 @@ __device__ __forceinline__ float mono_lg2(float2 q, float2 c) {
 }
 
 // Monopole kernel of panel j at a node: -log|q - c| / 2pi (the near pairs
-// subtract exactly this value).
+// subtract this value; where a near panel is part of a far cluster, its
+// moments stand for it to the series' remainder).
 __device__ __forceinline__ float mono32(float2 q, float2 c) { return kMonoLog2 * mono_lg2(q, c); }
 
 // corr[e][m] = (G_H 1_j)(q_{i,m}) - l_j mono32(q_{i,m}, c_j) for the near pair
@@ -917,6 +918,13 @@ void TwoLevel::plan_clusters(const std::vector<double> &cen, const Geometry &G) 
         double x, y, r;
     };
     std::vector<Node> nd;
+    // A cluster counts as at least eight units in the last place of the FP32
+    // positions wide: one panel alone (or panels at one point) has no radius,
+    // a node apart from it by less than a float would be "far" and, in
+    // floats, at distance zero.
+    double most = 0.0;
+    for (double c : cen) most = std::max(most, std::fabs(c));
+    const double resolved = std::max(0x1p-21 * most, 1e-30);
     auto add = [&](int lo, int hi, int child, int nchild) {
         double bx0 = 1e300, by0 = 1e300, bx1 = -1e300, by1 = -1e300, r2 = 0.0;
         for (int p = lo; p < hi; ++p) {
@@ -931,7 +939,7 @@ void TwoLevel::plan_clusters(const std::vector<double> &cen, const Geometry &G) 
             const double *c = &cen[2 * (size_t)h_mo_[p]];
             r2 = std::max(r2, (c[0] - x) * (c[0] - x) + (c[1] - y) * (c[1] - y));
         }
-        nd.push_back({lo, hi, child, nchild, x, y, std::sqrt(r2)});
+        nd.push_back({lo, hi, child, nchild, x, y, std::max(std::sqrt(r2), resolved)});
     };
     for (int lo = 0; lo < P; lo += kLeafPanels) add(lo, std::min(P, lo + kLeafPanels), -1, 0);
     n_leaves_ = int(nd.size());
@@ -963,7 +971,7 @@ void TwoLevel::plan_clusters(const std::vector<double> &cen, const Geometry &G) 
             stack.pop_back();
             const Node &n = nd[b];
             const double d = std::hypot(n.x - nd[t].x, n.y - nd[t].y) - rt;
-            if (d >= kClusterSep * n.r && d > 0.0) h_list_.push_back(b);
+            if (d >= kClusterSep * n.r) h_list_.push_back(b);
             else if (n.child < 0) near.push_back(b);
             else
                 for (int q = 0; q < n.nchild; ++q) stack.push_back(n.child + q);
@@ -982,8 +990,7 @@ void TwoLevel::plan_clusters(const std::vector<double> &cen, const Geometry &G) 
     h_geo_.resize(nd.size());
     h_range_.resize(nd.size());
     for (size_t b = 0; b < nd.size(); ++b) {
-        const double r = std::max(nd[b].r, 1e-12);   // one panel, or panels at one point
-        h_geo_[b] = make_float4((float)nd[b].x, (float)nd[b].y, (float)r, (float)(1.0 / r));
+        h_geo_[b] = make_float4((float)nd[b].x, (float)nd[b].y, (float)nd[b].r, (float)(1.0 / nd[b].r));
         h_range_[b] = make_int2(nd[b].lo, nd[b].hi);
     }
 }
