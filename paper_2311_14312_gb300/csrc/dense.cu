@@ -159,12 +159,16 @@ __device__ void dense_eval_body(double qx, double qy, bool active, const double 
 // consecutive pixels, kGridSets threads to each, every set its share of the
 // segments (each pixel alone would leave most of the GPU idle below a few
 // hundred thousand pixels); the sets' sums are added in order.  The frame's
-// origin is the middle of the run and its unit w, a power of two at least as
-// large as the drawing and the viewport, so that squares of distances are
-// normal floats on any canvas; the logarithms are then log(r / w), and log(w)
-// times the segments' weighted lengths is added in FP64.  Bound by FP32 issue, 450 instructions a
-// pair: 128^2 pixels of 5,120 segments in 1.86 ms on one GB300, 27.7 with the
-// pairs in FP64.
+// origin is the middle of the run and its unit w, a power of two of the size of
+// the drawing and the viewport, so that squares of distances are normal floats
+// on any canvas; the logarithms are then log(r / w), and log(w) times the
+// segments' weighted lengths is added in FP64.  A logarithm's error grows with
+// its size, so the unit is the typical distance, a quarter to half of the
+// extent: on three drawings (four closed curves, densities to 7,400) the
+// error against 113-bit sums is 1.2 to 2.3e-14 (rms; at most 2.3e-13), at four
+// times the unit 3.6 to 5.4e-14, in FP64 3.2 to 5.7e-14 (at most 2.3e-13).
+// Bound by FP32 issue, 450 instructions a pair: 128^2 pixels of 5,120 segments
+// in 1.86 ms on one GB300, 27.7 with the pairs in FP64.
 constexpr int kGridPixels = 64, kGridSets = 4;
 __global__ void __launch_bounds__(kGridPixels *kGridSets, 2)
 dense_eval_grid_kernel(const double *__restrict__ seg, const double *__restrict__ segw,
@@ -482,7 +486,7 @@ cudaError_t launch_dense_eval_grid(const DevGeom &G, const double *sbar, const d
         const double a = d ? vp.y0 : vp.x0, b = a + (d ? vp.height * vp.dy : vp.width * vp.dx);
         ext = std::max(ext, std::max({G.box[2 + d], a, b}) - std::min({G.box[d], a, b}));
     }
-    const double w = std::ldexp(1.0, ext > 0.0 && std::isfinite(ext) ? std::min(std::ilogb(ext) + 1, 1000) : 0);
+    const double w = std::ldexp(1.0, ext > 0.0 && std::isfinite(ext) ? std::min(std::ilogb(ext) - 1, 1000) : 0);
     unsigned blocks = (unsigned)((npix + kGridPixels - 1) / kGridPixels);
     dense_eval_grid_kernel<<<blocks, kGridPixels * kGridSets, 0, st>>>(G.seg.ptr, G.segw.ptr, sbar, mbar, G.S, vp, w,
                                                                     u); note_launch();
