@@ -64,8 +64,13 @@ typedef enum {
 /* How the layer-potential operator is applied. */
 typedef enum {
     DC_FORM_DENSE64 = 0,    /* plain form: dense FP64 operator rows (Eq. 19,
-                               27) and FP64 direct sums for pixels (A11)    */
-    DC_FORM_FMM64 = 1,      /* FP64 FMM on the non-uniform quadtree (Alg. 8) */
+                               27) and direct sums for pixels (A11): FP64 for
+                               points, for a viewport's pixels pairs of
+                               floats, as near to exact sums as FP64        */
+    DC_FORM_FMM64 = 1,      /* FMM on the non-uniform quadtree (Alg. 8) to
+                               FP64's accuracy: points in FP64, expansions,
+                               stored coefficients and pixels in pairs of
+                               floats                                       */
     DC_FORM_FMM32 = 2       /* chosen form: FP32 FMM with FP64 GMRES
                                (Arnoldi, least squares, outer residual)     */
 } dc_form;

@@ -286,8 +286,9 @@ static __global__ void __launch_bounds__(32 * kWarps) near_coef_kernel(NodeArgs<
 // a third float: in a leaf as wide as the canvas (hi, lo) drops up to five of
 // FP64's bits.  A pair's 2^-47 adds up over a leaf's list: up to kFfLeaf pieces
 // a leaf the operator is as close to the direct sum as with FP64 coefficients
-// (6.2e-12 of F_H x, 16 curves), with all 6,000 in one leaf it was 1.6e-11, so
-// larger leaves keep FP64.  Blocks stay resident and take every gridDim.x-th
+// (5.9e-13 of F_H x, 16 curves), with the 6,000 pieces of that drawing in a
+// few leaves (depth limits 1 and 2) it was 3.9e-11 and 1.6e-11, in FP64 2.2e-12
+// and 4.9e-13, so larger leaves keep FP64.  Blocks stay resident and take every gridDim.x-th
 // item, since each fills the tables once.
 // The build of a 200-curve drawing takes 11.1 ms instead of 12.7, curves to
 // image 21.7 instead of 24.2.

@@ -63,7 +63,7 @@ __device__ __forceinline__ unsigned char q8(double v) {
 // log(w) times the pieces' total weighted length, is added in FP64).  Bound by
 // FP32 issue: 450 instructions a pair and 100 a coefficient and channel
 // triple.  517 x 509 pixels of a 48-curve drawing (76 list-1 pieces and 7
-// list-3 cells a pixel) in 1.12 ms on one GB300, 9.95 with the pairs and
+// list-3 cells a pixel) in 1.05 ms on one GB300, 9.95 with the pairs and
 // expansions in FP64, whose pipe they saturated; the error against a 64-bit
 // direct sum is the same 1.6e-12 (the expansions' truncation).
 constexpr int kFfThreads = 64, kFfBlocksPerSM = 8;

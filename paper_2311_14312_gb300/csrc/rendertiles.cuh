@@ -17,9 +17,12 @@
 // points for 256 pixels instead, they cost an eighth, and with the four
 // pixels +-x +-y of a rectangle sharing the powers of z the polynomial takes
 // 2.5 instructions per term and pixel.  Bound by instruction issue; on one
-// GB300 the evaluation went from 3.00 to 1.03 ms there (27.6 to about 8 G lane
+// GB300 the evaluation went from 3.00 to 1.05 ms there (27.6 to about 8 G lane
 // instructions of pair, expansion and polynomial work), and 24 viewports up to
-// zoom 10^6 of the 2000-curve drawing (87 Mpixels) from 27 to 8.2 ms.
+// zoom 10^6 of the 2000-curve drawing (87 Mpixels) from 27 to 8.4 ms.  Against
+// 64-bit direct sums an image is off by 8e-8 (rms of the field; 1e-7 when every
+// pixel was evaluated directly), 2% of the time being for sums that keep what
+// large parts cancel (add_parts) and for a cut by channel.
 //
 // A block of four warps takes a rectangle: the warps share the sources of the
 // samples (lanes = samples), then the pixels (lanes = pixels; in a rectangle
