@@ -905,7 +905,19 @@ void TwoLevel::plan(const Geometry &G, int max_coarse) {
     n_leaves_ = 0;
     h_geo_.clear();
     h_far_.clear();
-    if (K_ == 1 && P >= kTreePanels) plan_clusters(cen, G);
+    if (K_ == 1 && P >= kTreePanels) {
+        // On a canvas so small that mono_lg2's bound on a distance shows, or
+        // squares of distances leave the normal floats, and on one so large
+        // that they might overflow, the sum stays direct.
+        double lo[2] = {cen[0], cen[1]}, hi[2] = {cen[0], cen[1]};
+        for (int j = 0; j < P; ++j)
+            for (int d = 0; d < 2; ++d) {
+                lo[d] = std::min(lo[d], cen[2 * j + d]);
+                hi[d] = std::max(hi[d], cen[2 * j + d]);
+            }
+        const double ext = std::max(hi[0] - lo[0], hi[1] - lo[1]);
+        if (ext >= 0x1p-36 && ext <= 0x1p40) plan_clusters(cen, G);
+    }
     planned_ = true;
 }
 

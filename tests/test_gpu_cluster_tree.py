@@ -2,6 +2,8 @@
 themselves against the definition (the coarse solution, whose FP32 inverse
 would hide them, is eliminated), and a node that coincides, in floats, with
 the only panel of a cluster outside its own."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -31,7 +33,8 @@ def _operators(O, d):
 
 def _apply(dcmod, d, v):
     import torch
-    ctx = dcmod.Context(form="fmm32", g=d.g, s_per_panel=d.s_per_panel, p=24, leaf_size=32)
+    ctx = dcmod.Context(form="fmm32", g=d.g, s_per_panel=d.s_per_panel, p=24, leaf_size=32,
+                        domain=(0.0, 0.0, float(d.ctrl[..., 0].max()), float(d.ctrl[..., 1].max())))
     ctx.build_drawing(d)
     info = ctx.precond_info()
     assert info["two_level"] == 1.0 and info["panels"] == d.n_panels
@@ -53,15 +56,21 @@ def _distance(dcmod, O, d):
     return np.linalg.norm(rhs - C @ y) / np.linalg.norm(w)
 
 
-@pytest.mark.parametrize("curves,per_curve", [(16, 128), (13, 159)])   # 2048, 2067 panels
-def test_cluster_sums_match_definition(dcmod, cuda_ok, oracle_mod, curves, per_curve):
+def _closed(curves, per_curve, scale):
+    d = make_closed_set(61, n_curves=curves, panels_per_curve=per_curve, g=4)
+    return dataclasses.replace(d, ctrl=d.ctrl * scale)
+
+
+@pytest.mark.parametrize("curves,per_curve,scale", [(16, 128, 1.0), (13, 159, 1.0),   # 2048, 2067 panels
+                                                    (13, 159, 2.0 ** -34), (13, 159, 2.0 ** -56)])
+def test_cluster_sums_match_definition(dcmod, cuda_ok, oracle_mod, curves, per_curve, scale):
     # Bound: as near as the direct sum, which takes over just below 2,048 panels, is on the same curves with
     # fewer panels, but for a factor of two (B enlarges the FP32 rounding of either; a separation of 1.5
     # instead of 2.5 would add terms that are off by 3e-3)
     O = oracle_mod
-    rel = _distance(dcmod, O, make_closed_set(61, n_curves=curves, panels_per_curve=per_curve, g=4))
-    direct = _distance(dcmod, O, make_closed_set(61, n_curves=curves, panels_per_curve=2047 // curves, g=4))
-    print(f"{curves * per_curve} panels: {rel:.2e}, direct {direct:.2e}")
+    rel = _distance(dcmod, O, _closed(curves, per_curve, scale))
+    direct = _distance(dcmod, O, _closed(curves, 2047 // curves, scale))
+    print(f"{curves * per_curve} panels, canvas {scale:g}: {rel:.2e}, direct {direct:.2e}")
     assert rel <= 2 * direct
 
 
